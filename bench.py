@@ -342,7 +342,7 @@ def run_awo(args, R: Ranks):
     # velocity and mipmap: one launch for both and levels 1..6, one per further level (velocity alone
     # without a mipmap)
     lod_launches = 1 if w.lod_levels <= 1 else 1 + max(w.lod_levels - 1 - 6, 0)
-    launches_per_step = 1 + 3 + 2 + lod_launches
+    launches_per_step = 1 + 3 + 3 + lod_launches
 
     peaks_probe = _probe_peaks(torch, awo)
     clocks = ClockSampler(R.local)

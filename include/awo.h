@@ -293,8 +293,8 @@ awo_status awo_dem_gather_path(const float* d_h, awo_grid g, void* stream, int32
 awo_status awo_simulate_time_kernel(void* ev_start, void* ev_stop);
 
 /*
- * c (batched). Particle trajectories for many regions in one persistent
- * launch (the paper's workflow re-run for many regions and parameter sets;
+ * c (batched). Particle trajectories for many regions in one call without a
+ * gap between them (the paper's workflow re-run for many regions and parameter sets;
  * Sec. 5.2 lets the user change the parameters interactively).  Every request
  * gets exactly the rasters and statistics that awo_simulate would give it
  * alone (same formulas, same Philox streams; reductions are
@@ -308,7 +308,7 @@ awo_status awo_simulate_time_kernel(void* ev_start, void* ev_stop);
  *  - d_stats: device array of n_req awo_sim_stats, overwritten (nullable).
  *  - Workspace: awo_simulate_batched_workspace_bytes(reqs, n_req) bytes,
  *    16-byte aligned, contents undefined on entry and exit.
- * The request table travels in the kernel's parameter block: the call makes
+ * The request table travels in the kernels' parameter blocks: the call makes
  * no host-to-device copy and no allocation.
  */
 #define AWO_BATCH_MAX 128
@@ -328,12 +328,11 @@ typedef struct {
 /* Launch shape of the batched particle kernel (the autotuner's search space).
  *   threads_per_block: 64, 128 or 256 (0 = 128)
  *   group_particles:   particles a warp takes per fetch, 32 .. 65536 (0 = chosen
- *                      per launch: about all particles / (4 x the grid's warps),
- *                      rounded down to a multiple of 32, within 32 .. 1024)
- *   refill: AWO_REFILL_LANE -- ended lanes take the next particles while the
- *           warp's other lanes keep moving, once the idle lanes add up to 12
- *           idle lane-iterations (trajectory per thread, continuously
- *           refilled);
+ *                      per request: about its particles / (16 x the launch's
+ *                      warps), rounded down to a multiple of 32, within 32 .. 1024)
+ *   refill: AWO_REFILL_LANE -- lanes whose particle has ended take another one
+ *           while the warp's other lanes keep moving (trajectory per thread,
+ *           continuously refilled);
  *           AWO_REFILL_WARP -- a warp starts 32 particles together and takes
  *           the next 32 only when all have ended (trajectories per warp, in
  *           lock-step batches). */

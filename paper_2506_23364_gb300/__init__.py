@@ -374,7 +374,7 @@ def awo_simulate_batched_workspace_bytes(reqs) -> int:
 
 def awo_simulate_batched(reqs, ws: torch.Tensor, tuning: Tuning | None = None, stats: torch.Tensor | None = None,
                          stream=None):
-    """One persistent launch over all regions; stats: int64 [n_req, 6] on the device."""
+    """The particles of all regions in one call; stats: int64 [n_req, 6] on the device."""
     arr = _req_array(reqs)
     sp = _dev(stats, torch.int64, 6 * len(arr), "stats") if stats is not None else None
     _check(lib().awo_simulate_batched(arr, len(arr), ctypes.byref(tuning) if tuning is not None else None, sp,

@@ -2,6 +2,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 
 #include "awo.h"
@@ -57,6 +58,14 @@ inline bool sim_params_ok(const awo_sim_params* p, float cs)
     if (!(kD < 1.0f)) return false;
     if ((p->flags & ~AWO_SIM_CLEAR_OUTPUTS) != 0u) return false;
     return true;
+}
+
+// R 2^-23 for the particle kernels' random part, or NaN when that product is
+// not exact (R so small that it is subnormal): they take the general form then.
+inline float scaled_randomness(float R)
+{
+    const float r = R * 0x1p-23f;
+    return r * 0x1p23f == R ? r : NAN;
 }
 
 // Size of the release texture at 2^r times the resolution of grid g

@@ -4,41 +4,47 @@
 //  * Persistent kernel, one lane per particle.  The particles are numbered
 //    cell-major (start record, then particle j); a warp takes a chunk of
 //    consecutive particles at a time from a global counter (one atomic per
-//    chunk) and walks it with a warp-uniform cursor; a lane is refilled the
-//    moment its particle ends, so lanes never idle behind a long particle of
-//    the same warp.  The chunk size (32 .. 1024 particles) follows from the
-//    particle count and the grid, so that a release list of a few cells is
-//    still spread over many warps.  The start records are in a processing
-//    order that spreads consecutive blocks of release cells over the grid
-//    (order_slot): the lanes of a warp work on neighbouring cells, while the
-//    warps of the GPU work all over the grid and its memory partitions.
-//  * One integer division per chunk and none per particle: the cursor
-//    carries (release-list entry, j), and the start record holds the cell's
-//    coordinates.
-//  * A particle starts at refill time from the 16-byte start record of its
-//    release cell (position, height, first direction), written by a prologue
-//    kernel that also records the release visits of all N particles of the
-//    cell with one reduction.  Each loop iteration is then two moves and
-//    their visits from one Philox block (moves n and n + 1 take words 0-1 and
-//    2-3 of block n >> 1; live lanes are always at an even n there) --
-//    direction from the footprint kept in registers, step, footprint and
-//    energy at the new position, record -- written without data-dependent
-//    branches (selects and predicated reductions), so a warp runs one
-//    instruction stream.
+//    chunk) and walks it with a warp-uniform cursor (one integer division per
+//    chunk, none per particle).  The chunk size (32 .. 1024 particles) follows
+//    from the particle count and the grid, so that a release list of a few
+//    cells is still spread over many warps.  The start records are in a
+//    processing order that spreads consecutive blocks of release cells over
+//    the grid (order_slot): the lanes of a warp work on neighbouring cells,
+//    while the warps of the GPU work all over the grid and its memory
+//    partitions.
+//  * 32 particles start together and make their first two moves ("fresh"
+//    pair); the survivors then run beside survivors of earlier starts, and
+//    lanes whose particle ends take over a waiting one from the warp's pool in
+//    shared memory (awo_particle.cuh, run_particles).
+//  * A particle starts from the 16-byte start record of its release cell
+//    (position, height, first move vector before its random part), written by
+//    a prologue kernel that also records the release visits of all N
+//    particles of the cell with one reduction.  Each loop iteration is two
+//    moves and their visits from one Philox block (moves n and n + 1 take
+//    words 0-1 and 2-3 of block n >> 1; live lanes are always at an even n
+//    there) -- direction from the gradient kept in registers, step, footprint
+//    and energy at the new position, record -- written without data-dependent
+//    branches.
 //  * Visits go to the rasters as fire-and-forget reductions (RED.ADD on the
-//    count, RED.MAX on the bits of the non-negative energy), one pair per
-//    lane: measured on GB300, merging the lanes of a warp that hit the same
-//    cell (__match_any_sync + __reduce_max_sync) costs more issue slots than
-//    the L2 spends on the duplicate reductions.
-//  * Philox4x32-10 round keys are computed once on the host and read from the
-//    kernel's parameter bank.
+//    count, RED.MAX on the bits of the non-negative energy, the latter only if
+//    it can raise the maximum, where looking pays: check_pays).  Merging the
+//    lanes of a warp that hit the same cell (__match_any_sync, at the first
+//    move, at both moves of a fresh pair or at every move) was slower wherever
+//    the look is taken (8192^2 18.2 against 17.6 ms, at every move 19.6).
 //  * On grids of at least 2^20 cells the 2x2 footprint of a move is one
 //    texture gather through a texture object that views the DEM's words
 //    (clamp addressing is the footprint clamp; indices and weights are still
 //    computed here), in place of four loads, their addresses and clamps.
 //  * Arithmetic is FP32 with explicit round-to-nearest intrinsics: no fused
-//    multiply-add, IEEE sqrt and reciprocal, so every particle follows the
-//    formulas of awo.h bit for bit.
+//    multiply-add that changes a rounding, IEEE sqrt and reciprocal, so every
+//    particle follows the formulas of awo.h bit for bit.
+//  * What bounds it: issue on the 8192^2 workload (82% of issue slots; 151
+//    warp instructions per move of a warp, from 222), the visits' traffic to
+//    the L2 and the footprint gathers' latency on the long-trajectory ones
+//    (2048^2: 73% of issue slots, L2 62%, from 67% and 72%).  Measured and not
+//    kept: the paired arithmetic of a move in packed FP32 (fma.rn.f32x2, its
+//    products kept separately rounded by an addend of -0 that the compiler
+//    cannot see): 17.1 against 17.2 ms; 40 registers for 12 blocks an SM: 17.4.
 #include <math.h>
 #include <string.h>
 
@@ -48,50 +54,12 @@
 
 namespace awo {
 
-struct SimWorkspace {
-    unsigned long long next_item;  // global work counter, in particles
-    unsigned long long stats[6];   // total_steps, n_traj, n_exited, n_capped, n_stopped, n_rejected
-    unsigned long long pad;
-};
-static_assert(sizeof(SimWorkspace) == 64, "workspace layout");
-
-struct SimArgs {
-    // request constants (names read by AWO_MOVE_WORDS)
-    const float* h;
-    uint32_t* count;
-    float* maxe;
-    int W, H;
-    float Wm1, Hm1;        // W-1, H-1 as floats (exact for W, H <= 2^24)
-    float P, oneP, R, s;   // persistence, 1-P, randomness, step in cells
-    float kD, muD;         // drag_k*D, mu*D  (D = s*cell_size)
-    uint32_t max_steps;
-    KeysTable keys;        // Philox round keys
-    // work
-    const uint32_t* cells;
-    const uint32_t* n_cells_dev;
-    uint32_t n_cells_max;
-    uint32_t n_grid;       // W*H
-    uint32_t N;
-    TexelGeom tg;          // release texture (texel mode only)
-    SimWorkspace* ws;
-    void* starts;          // one start record per release-list entry (CellStart or TexelStart)
-    cudaTextureObject_t tex;  // texture view of h (the gathers of k_simulate<_, true>), or 0
-};
-
-constexpr int SIM_THREADS = 128;
+constexpr int SIM_THREADS = 128, SIM_THREADS_MAX = 256;
 constexpr uint32_t SIM_CHUNK_MAX = 1024;  // particles per global fetch, at most
 // fetches a warp makes on an even split, at least: chunks of neighbouring
 // cells carry similar work, so few large chunks leave some warps with much
 // more of it (2048^2 workload: 4 -> 16 chunks a warp, 1.80 -> 1.72 ms)
 constexpr uint32_t SIM_CHUNKS_PER_WARP = 16;
-// A warp refills its idle lanes once they add up to SIM_REFILL_IDLE idle
-// lane-iterations since its last refill (or when every lane is idle): a
-// refill round costs issue slots whether it starts one particle or thirty,
-// so refilling for a single idle lane wastes slots, and waiting too long
-// leaves lanes idle.  Measured on GB300 (8192^2 particle kernel, ms, with the
-// counters folded per particle): 1 -> 20.61, 2 -> 20.50, 3 -> 20.46,
-// 4 -> 20.46, 6 -> 20.46, 8 -> 20.54, 12 -> 20.67, 16 -> 20.88.
-constexpr uint32_t SIM_REFILL_IDLE = 4;
 
 __device__ __forceinline__ uint32_t release_count(const SimArgs& a)
 {
@@ -133,12 +101,14 @@ __global__ void __launch_bounds__(256) k_sim_starts(const __grid_constant__ SimA
         const uint32_t entry = __ldg(a.cells + ci);
         bool ok;
         if (TEXELS) {
-            const TexelStart st = texel_start(a.h, a.W, a.H, a.tg, entry);
+            TexelStart st = texel_start(a.h, a.W, a.H, a.tg, entry);
+            first_vector(st, a.P, a.oneP);
             ok = st.t != ~0u;
             if (ok) atomicAdd(a.count + st.vcell, a.N);
             static_cast<TexelStart*>(a.starts)[slot] = st;
         } else {
-            const CellStart st = cell_start(a.h, a.W, a.H, a.n_grid, entry);
+            CellStart st = cell_start(a.h, a.W, a.H, a.n_grid, entry);
+            first_vector(st, a.P, a.oneP);
             ok = st.xy != ~0u;
             if (ok) atomicAdd(a.count + entry, a.N);
             static_cast<CellStart*>(a.starts)[slot] = st;
@@ -160,105 +130,131 @@ __global__ void __launch_bounds__(256) k_sim_starts(const __grid_constant__ SimA
     }
 }
 
-template <bool TEXELS, bool TEX>
-__global__ void __launch_bounds__(SIM_THREADS) k_simulate(const __grid_constant__ SimArgs a)
+// The particle kernel, in two instances per kind of record and footprint:
+// with and without the look at a cell's maximum (CHECK).  Which one runs
+// depends on the release count, which the host does not know, so both are
+// launched and one of them ends at once (as one kernel that holds both loops,
+// or with the choice as a predicate, the 8192^2 workload took 2% more).
+//
+// Every launch lets the next one start as soon as its blocks are resident
+// (programmatic dependent launch), so the blocks of a batch's next request
+// fill the SMs as this one's warps run out of particles.  The last block of a
+// launch does nothing but wait for the launch before it, so that a launch is
+// complete only when all before it are, and what follows on the stream is
+// ordered after every one.  (The same wait at the end of a working block cost
+// 8 registers and 5% on the 8192^2 workload.)
+template <bool TEXELS, bool TEX, bool CHECK>
+__global__ void __launch_bounds__(SIM_THREADS_MAX) k_simulate(const __grid_constant__ SimArgs a)
 {
-    constexpr int kGather = TEX ? 1 : 0;  // footprints by texture gather or loads (read by AWO_MOVE_WORDS)
-    const int lane = threadIdx.x & 31;
-    const unsigned lane_lt = (1u << lane) - 1u;
-    const uint32_t n_cells = release_count(a);
-
-    // particles in all, and the chunk a warp takes per fetch: a multiple of
-    // 32 in [32, SIM_CHUNK_MAX], about total / (warps * SIM_CHUNKS_PER_WARP)
-    const unsigned long long total = (unsigned long long)n_cells * a.N;
-    const unsigned long long warps = (unsigned long long)gridDim.x * (blockDim.x >> 5);
-    unsigned long long chunk = total / (warps * SIM_CHUNKS_PER_WARP);
-    chunk = chunk < 32ull ? 32ull : (chunk > SIM_CHUNK_MAX ? (unsigned long long)SIM_CHUNK_MAX : chunk);
-    chunk &= ~31ull;
-
-    // warp-uniform cursor: next particle (t, and as (entry, j)) and the end of the chunk
-    unsigned long long cur_t = 0ull, end_t = 0ull;
-    uint32_t cur_ci = 0, cur_j = 0;
-    bool exhausted = (total == 0ull);
-    uint32_t idle_acc = 0u;  // idle lane-iterations since the last refill (warp-uniform)
-
-    AWO_LANE_STATE
-
-    while (true) {
-        // ---- refill idle lanes (once they add up to SIM_REFILL_IDLE) --------
-        const unsigned idle = __ballot_sync(0xffffffffu, !live);
-        idle_acc += (uint32_t)__popc(idle);
-        if (idle != 0u && idle_acc >= SIM_REFILL_IDLE && !exhausted) {
-            idle_acc = 0u;
-            if (cur_t >= end_t) {
-                unsigned long long base = 0;
-                if (lane == 0) base = atomicAdd(&a.ws->next_item, chunk);
-                base = __shfl_sync(0xffffffffu, base, 0);
-                exhausted = base >= total;
-                if (!exhausted) {
-                    cur_t = base;
-                    end_t = min(total, base + chunk);
-                    cur_ci = (uint32_t)(base / a.N);  // one division per chunk
-                    cur_j = (uint32_t)(base - (unsigned long long)cur_ci * a.N);
-                }
-            }
-            if (!exhausted) {
-                // particles left in the chunk (capped at 32)
-                const unsigned long long left = end_t - cur_t;
-                const unsigned avail = left < 32ull ? (unsigned)left : 32u;
-                const unsigned want = (unsigned)__popc(idle);
-                const unsigned take = want < avail ? want : avail;
-                const unsigned rank = (unsigned)__popc(idle & lane_lt);
-                const bool mine = ((idle >> lane) & 1u) && rank < take;
-                uint32_t ci = cur_ci, jj = cur_j;
-                advance(ci, jj, rank < take ? rank : 0u, a.N);
-                uint4 st = make_uint4(~0u, 0u, 0u, 0u), st1 = make_uint4(0u, 0u, 0u, 0u);
-                if (TEXELS) {
-                    if (mine) {
-                        st = __ldg(reinterpret_cast<const uint4*>(a.starts) + 2u * ci);
-                        st1 = __ldg(reinterpret_cast<const uint4*>(a.starts) + 2u * ci + 1u);
-                    }
-                } else {
-                    if (mine) st = __ldg(reinterpret_cast<const uint4*>(a.starts) + ci);
-                }
-                // entries outside the grid are skipped here and counted by the prologue
-                const bool ok = mine && st.x != ~0u;
-                AWO_FOLD_LANE(mine, a.max_steps);
-                if (TEXELS)
-                    AWO_LANE_START_TEXEL(ok, st, st1, jj);
-                else
-                    AWO_LANE_START(ok, st, jj, a.W);
-                my_traj += ok ? 1u : 0u;  // particles are counted when they start
-                live = live || ok;
-                advance(cur_ci, cur_j, take, a.N);
-                cur_t += take;
-            }
-        }
-        if (__ballot_sync(0xffffffffu, live) == 0u) {
-            if (exhausted) break;
-            continue;
-        }
-        AWO_MOVE_PAIR(a, a.keys);
+    extern __shared__ uint32_t s_pool[];  // POOL_WORDS per warp
+    asm volatile("griddepcontrol.launch_dependents;");
+    const uint32_t blocks = gridDim.x - 1u;
+    if (blockIdx.x == blocks) {
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        return;
     }
-    AWO_FOLD_LANE(true, a.max_steps);
-    AWO_FLUSH_COUNTERS(a.ws->stats);
+    const unsigned long long total = (unsigned long long)release_count(a) * a.N;
+    const bool check = a.check ? *a.check != 0u
+                               : check_pays(total, (unsigned long long)blocks * blockDim.x, a.n_grid);
+    const uint32_t warp = threadIdx.x >> 5;
+    // a few particles: one warp a block, so that they spread over the SMs
+    // (parabola, 6144 particles: 149 -> 135 us)
+    if (check == CHECK && total > 32ull * blocks * warp) {
+        // particles of entries inside the grid (the prologue has counted the others)
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            const unsigned long long run = total - a.ws->stats[5];
+            a.ws->stats[1] = run;
+            atomicAdd(&a.ws->stats[4], run);
+        }
+        // particles a warp takes per fetch: a multiple of 32 in [32,
+        // SIM_CHUNK_MAX], about total / (warps * SIM_CHUNKS_PER_WARP)
+        const unsigned long long even = total / ((unsigned long long)blocks * (blockDim.x >> 5) * SIM_CHUNKS_PER_WARP);
+        uint32_t chunk = even > SIM_CHUNK_MAX ? SIM_CHUNK_MAX : max((uint32_t)even & ~31u, 32u);
+        if (a.group) chunk = a.group;
+        run_particles<TEXELS, TEX ? 1 : 0, CHECK>(a, total, chunk, a.min_idle, &a.ws->next_item, a.ws->stats,
+                                                  s_pool + warp * POOL_WORDS);
+    }
 }
 
-template <bool TEXELS, bool TEX>
-static int sim_blocks_per_sm()
+template <bool TEXELS, bool TEX, bool CHECK>
+static awo_status launch_instance(const SimArgs& a, int threads, bool after_particles, cudaStream_t s)
 {
-    static int cached[64] = {0};
+    static int cached[64][3];  // resident blocks per SM, by device and block size (a race writes the same value)
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 64) dev = 0;
-    if (cached[dev] == 0) {
+    const size_t shared = (size_t)(threads / 32) * POOL_WORDS * sizeof(uint32_t);
+    int& per_sm = cached[dev][threads == 64 ? 0 : (threads == 128 ? 1 : 2)];
+    if (per_sm == 0) {
         int b = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_simulate<TEXELS, TEX>, SIM_THREADS, 0) != cudaSuccess ||
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_simulate<TEXELS, TEX, CHECK>, threads, shared) !=
+                cudaSuccess ||
             b < 1)
             b = 1;
-        cached[dev] = b;
+        per_sm = b;
     }
-    return cached[dev];
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3((unsigned)(sm_count() * per_sm + 1));
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = shared;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = after_particles ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, k_simulate<TEXELS, TEX, CHECK>, a) == cudaSuccess ? launch_status() : AWO_ECUDA;
+}
+
+template <bool TEXELS, bool TEX>
+static awo_status launch_both(const SimArgs& a, int threads, bool after_particles, cudaStream_t s)
+{
+    const awo_status st = launch_instance<TEXELS, TEX, true>(a, threads, after_particles, s);
+    return st != AWO_OK ? st : launch_instance<TEXELS, TEX, false>(a, threads, true, s);
+}
+
+awo_status launch_particles(const SimArgs& a, int threads, bool after_particles, cudaStream_t s)
+{
+    if (a.tg.texels)
+        return a.tex ? launch_both<true, true>(a, threads, after_particles, s)
+                     : launch_both<true, false>(a, threads, after_particles, s);
+    return a.tex ? launch_both<false, true>(a, threads, after_particles, s)
+                 : launch_both<false, false>(a, threads, after_particles, s);
+}
+
+void sim_constants(SimArgs& a, const float* d_h, awo_grid g, const awo_sim_params* p, uint32_t* d_count, float* d_maxe,
+                   cudaStream_t s)
+{
+    memset(&a, 0, sizeof(a));
+    // each one FP32 rounding in the documented order
+    const float D = p->step_scale * g.cell_size;
+    a.h = d_h;
+    a.count = d_count;
+    a.maxe = d_maxe;
+    a.W = g.width;
+    a.H = g.height;
+    a.n_grid = (uint32_t)cells_of(g);
+    a.Wm1 = (float)(g.width - 1);
+    a.Hm1 = (float)(g.height - 1);
+    a.P = p->persistence;
+    a.oneP = 1.0f - p->persistence;
+    a.R = p->randomness;
+    a.R23 = scaled_randomness(p->randomness);
+    a.s = p->step_scale;
+    a.kD = p->drag_k * D;
+    a.muD = p->mu * D;
+    a.N = p->traj_per_cell;
+    a.max_steps = p->max_steps;
+    a.keys = philox_keys(p->seed);
+    int64_t wr = 0, hr = 0;
+    release_texture_dims(g, p->release_log2, &wr, &hr);  // checked by sim_params_ok
+    a.tg.Wr = (uint32_t)wr;
+    a.tg.n_tex = (uint32_t)(wr * hr);
+    a.tg.scale = ldexpf(1.0f, -p->release_log2);
+    a.tg.texels = p->release_log2 != 0 ? 1u : 0u;
+    a.tex = dem_texture(d_h, g, s);
+    a.min_idle = 1u;
 }
 
 // Texture views of DEM buffers for the gathers of k_simulate: a texture
@@ -386,45 +382,14 @@ extern "C" awo_status awo_simulate(const float* d_h, awo_grid g, const uint32_t*
         if (cudaMemsetAsync(d_maxe, 0, bytes, s) != cudaSuccess) return AWO_ECUDA;
     }
 
-    // host-side constants, each one FP32 rounding in the documented order
-    const float D = p->step_scale * g.cell_size;
     SimArgs a;
-    a.h = d_h;
+    sim_constants(a, d_h, g, p, d_count, d_maxe, s);
     a.cells = d_cells;
     a.n_cells_dev = d_n_cells;
     a.n_cells_max = n_cells_max;
-    a.W = g.width;
-    a.H = g.height;
-    a.n_grid = (uint32_t)cells_of(g);
-    a.Wm1 = (float)(g.width - 1);
-    a.Hm1 = (float)(g.height - 1);
-    a.P = p->persistence;
-    a.oneP = 1.0f - p->persistence;
-    a.R = p->randomness;
-    a.s = p->step_scale;
-    a.kD = p->drag_k * D;
-    a.muD = p->mu * D;
-    a.N = p->traj_per_cell;
-    a.max_steps = p->max_steps;
-    uint32_t k0 = (uint32_t)(p->seed & 0xffffffffu), k1 = (uint32_t)(p->seed >> 32);
-    for (int r = 0; r < 10; ++r) {
-        a.keys.k0[r] = k0;
-        a.keys.k1[r] = k1;
-        k0 += 0x9E3779B9u;  // Weyl key schedule of Philox4x32
-        k1 += 0xBB67AE85u;
-    }
-    a.count = d_count;
-    a.maxe = d_maxe;
     a.ws = ws;
     a.starts = static_cast<char*>(d_ws) + starts_offset();
-    int64_t wr = 0, hr = 0;
-    release_texture_dims(g, p->release_log2, &wr, &hr);  // checked by sim_params_ok
-    a.tg.Wr = (uint32_t)wr;
-    a.tg.n_tex = (uint32_t)(wr * hr);
-    a.tg.scale = ldexpf(1.0f, -p->release_log2);
-    const bool texels = p->release_log2 != 0;
-
-    a.tex = dem_texture(d_h, g, s);
+    const bool texels = a.tg.texels != 0u;
 
     if (a.N > 0 && n_cells_max > 0 && a.max_steps == 0u) {  // every particle capped at its release visit
         const unsigned pro_blocks = stream_blocks((int64_t)n_cells_max, 256);
@@ -436,26 +401,14 @@ extern "C" awo_status awo_simulate(const float* d_h, awo_grid g, const uint32_t*
         if (st != AWO_OK) return st;
     } else if (a.N > 0 && n_cells_max > 0) {
         const unsigned pro_blocks = stream_blocks((int64_t)n_cells_max, 256);
-        const unsigned sms = (unsigned)sm_count();
         if (texels)
             k_sim_starts<true><<<pro_blocks, 256, 0, s>>>(a);
         else
             k_sim_starts<false><<<pro_blocks, 256, 0, s>>>(a);
         if (ev_start && cudaEventRecord(ev_start, s) != cudaSuccess) return AWO_ECUDA;
-        if (texels) {
-            if (a.tex)
-                k_simulate<true, true><<<sms * sim_blocks_per_sm<true, true>(), SIM_THREADS, 0, s>>>(a);
-            else
-                k_simulate<true, false><<<sms * sim_blocks_per_sm<true, false>(), SIM_THREADS, 0, s>>>(a);
-        } else {
-            if (a.tex)
-                k_simulate<false, true><<<sms * sim_blocks_per_sm<false, true>(), SIM_THREADS, 0, s>>>(a);
-            else
-                k_simulate<false, false><<<sms * sim_blocks_per_sm<false, false>(), SIM_THREADS, 0, s>>>(a);
-        }
+        const awo_status launched = launch_particles(a, SIM_THREADS, false, s);
+        if (launched != AWO_OK) return launched;
         if (ev_stop && cudaEventRecord(ev_stop, s) != cudaSuccess) return AWO_ECUDA;
-        awo_status st = launch_status();
-        if (st != AWO_OK) return st;
     } else if (ev_start) {  // no particle kernel: an empty interval after the call's work
         if (cudaEventRecord(ev_start, s) != cudaSuccess || cudaEventRecord(ev_stop, s) != cudaSuccess)
             return AWO_ECUDA;
