@@ -137,6 +137,8 @@ def lib() -> ctypes.CDLL:
         "awo_simulate": (st, [vp, Grid, vp, vp, u32, ctypes.POINTER(SimParams), vp, vp, vp, vp, sz, vp]),
         "awo_finalize": (st, [vp, Grid, f32, vp, vp]),
         "awo_normals_u16": (st, [vp, Grid, f32, vp, vp, vp, vp, vp]),
+        "awo_normals_release": (st, [vp, Grid, vp, vp, vp, f64, f64, vp, vp, vp, vp, sz, vp]),
+        "awo_normals_u16_release": (st, [vp, Grid, f32, vp, vp, vp, vp, f64, f64, vp, vp, vp, vp, sz, vp]),
         "awo_overlay_lod": (st, [vp, vp, Grid, i32, vp, vp, vp]),
         "awo_finalize_lod": (st, [vp, vp, Grid, f32, i32, vp, vp, vp, vp]),
         "awo_simulate_batched_workspace_bytes": (sz, [vp, i32]),
@@ -243,6 +245,27 @@ def awo_release(tan2: torch.Tensor, g: Grid, slope_lo_deg: float, slope_hi_deg: 
                              _dev(mask, torch.uint8, c, "mask"), _dev(cells, cells.dtype, c, "cells"),
                              _dev(n, n.dtype, 1, "n"), _dev(ws, torch.uint8, None, "ws"), ws.numel(),
                              _stream(stream)), "awo_release")
+
+
+def awo_terrain(src: torch.Tensor, g: Grid, scale: float | None, h: torch.Tensor, normal, tan2: torch.Tensor, slope_deg,
+                slope_lo_deg: float, slope_hi_deg: float, mask, cells: torch.Tensor, n: torch.Tensor, ws: torch.Tensor,
+                stream=None):
+    """awo_normals_u16_release (src: uint16 heights, decoded into h) or, with
+    scale None, awo_normals_release (src: FP32 heights; h is not used)."""
+    c = g.cells
+    if cells.dtype not in (torch.int32, torch.uint32) or n.dtype not in (torch.int32, torch.uint32):
+        raise TypeError("cells and n must be int32 or uint32")
+    outs = (_dev(normal, torch.float32, 3 * c, "normal"), _dev(tan2, torch.float32, c, "tan2"),
+            _dev(slope_deg, torch.float32, c, "slope_deg"), slope_lo_deg, slope_hi_deg,
+            _dev(mask, torch.uint8, c, "mask"), _dev(cells, cells.dtype, c, "cells"), _dev(n, n.dtype, 1, "n"),
+            _dev(ws, torch.uint8, None, "ws"), ws.numel(), _stream(stream))
+    if scale is None:
+        _check(lib().awo_normals_release(_dev(src, torch.float32, c, "h"), g, *outs), "awo_normals_release")
+        return
+    if src.dtype not in (torch.uint16, torch.int16):
+        raise TypeError("q must be uint16 (or int16 bits)")
+    _check(lib().awo_normals_u16_release(_dev(src, src.dtype, c, "q"), g, scale, _dev(h, torch.float32, c, "h"), *outs),
+           "awo_normals_u16_release")
 
 
 def awo_release_from_mask(mask: torch.Tensor, g: Grid, cells: torch.Tensor, n: torch.Tensor, ws: torch.Tensor,

@@ -106,18 +106,30 @@ inline bool sim_params_ok(const awo_sim_params* p, awo_grid g)
 // a's sign); otherwise negative a and -0 take the intrinsic.
 // awo_selftest_div_rn compares this function with the intrinsic on the
 // running GPU.
+constexpr uint32_t DIV_LOW = 0x21800000u, DIV_HIGH = 0x5d800000u;  // bits of 2^-60, 2^60
+
+// In that range, or for a = 0 (where -0 gives +0).
+__device__ __forceinline__ float div_rn_mid(float a, float b, float y)
+{
+    const float q0 = __fmul_rn(a, y);
+    const float q1 = __fmaf_rn(__fmaf_rn(-b, q0, a), y, q0);
+    return __fmaf_rn(__fmaf_rn(-b, q1, a), y, q1);
+}
+
+// q, of a's sign or zero, with a's sign.
+__device__ __forceinline__ float with_sign(float q, float a)
+{
+    return __uint_as_float(__float_as_uint(q) | (__float_as_uint(a) & 0x80000000u));
+}
+
 template <bool SIGNED = false>
 __device__ __forceinline__ float div_rn_by_rcp(float a, float b, float y)
 {
     const uint32_t ab = __float_as_uint(a) & (SIGNED ? 0x7fffffffu : 0xffffffffu);
-    const bool fast = (ab == 0u || (ab >= 0x21800000u && ab <= 0x5d800000u)) &&  // |a|: 0 or [2^-60, 2^60]
-                      (b >= 0x1p-60f && b <= 0x1p60f);
+    const bool fast = (ab == 0u || (ab >= DIV_LOW && ab <= DIV_HIGH)) && (b >= 0x1p-60f && b <= 0x1p60f);
     if (!fast) return __fdiv_rn(a, b);
-    const float m = __uint_as_float(ab);
-    const float q0 = __fmul_rn(m, y);
-    const float q1 = __fmaf_rn(__fmaf_rn(-b, q0, m), y, q0);
-    const float q2 = __fmaf_rn(__fmaf_rn(-b, q1, m), y, q1);
-    return SIGNED ? __uint_as_float(__float_as_uint(q2) | (__float_as_uint(a) & 0x80000000u)) : q2;
+    const float q = div_rn_mid(__uint_as_float(ab), b, y);
+    return SIGNED ? with_sign(q, a) : q;
 }
 #endif
 

@@ -72,8 +72,9 @@ __global__ void k_decode_u16(const uint16_t* __restrict__ q, int64_t n, float sc
 // cells of a row (no 64-bit division: a 32-bit item index splits into row and
 // run).  When rows are 16-byte aligned (W % 4 == 0 and aligned buffers) the
 // run's heights, the rows above and below and the outputs move as float4;
-// the two horizontal neighbours outside the run are scalar loads (L1 hits).
-// Otherwise each cell is handled alone with the same arithmetic.
+// the two horizontal neighbours outside the run are scalar loads (L1 hits)
+// (k_normals_tiles).  Otherwise each cell is handled alone with the same
+// arithmetic (k_normals).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void normal_of(float gx, float gy, float& nx, float& ny, float& nz, float& t2)
 {
@@ -86,7 +87,7 @@ __device__ __forceinline__ void normal_of(float gx, float gy, float& nx, float& 
 
 __device__ __forceinline__ float slope_deg_of(float t2) { return atanf(sqrtf(t2)) * 57.295779513082320876f; }
 
-// Heights for k_normals: FP32 metres, or (FROM_U16) uint16 words decoded
+// Heights for the normals: FP32 metres, or (FROM_U16) uint16 words decoded
 // exactly as k_decode_u16 does, h = (float)q * scale.
 template <bool FROM_U16>
 struct HeightSrc {
@@ -111,82 +112,143 @@ struct HeightSrc {
     }
 };
 
-// FROM_U16: the heights are decoded from uint16 words and also written to
-// h_out (each thread writes the cells of its run), so a0 and a1 take one
-// pass: awo_decode_u16 followed by awo_normals, without re-reading h.
+// The buffers and constants of one normals pass.  h_out (FROM_U16): the
+// decoded heights, each written by the thread of its run, so a0 and a1 take
+// one pass: awo_decode_u16 followed by awo_normals, without re-reading h.
 template <bool FROM_U16>
-__global__ void __launch_bounds__(256) k_normals(const HeightSrc<FROM_U16> h, int W, int H, float cs,
-                                                 float* __restrict__ nrm, float* __restrict__ tan2,
-                                                 float* __restrict__ slope_deg, float* __restrict__ h_out, bool vec4)
+struct NormalsArgs {
+    HeightSrc<FROM_U16> h;
+    int W, H;
+    float cs;
+    float* nrm;        // three planes, or null
+    float* tan2;       // or null
+    float* slope_deg;  // or null
+    float* h_out;
+};
+
+// Divisions of the finite differences by cs and 2 cs: div_rn_by_rcp, = __fdiv_rn.
+struct SpanDiv {
+    float den1, den2, rden1, rden2;
+};
+
+__device__ __forceinline__ SpanDiv span_div(float cs)
 {
+    const float cs2 = __fmul_rn(cs, 2.0f);
+    return SpanDiv{cs, cs2, __frcp_rn(cs), __frcp_rn(cs2)};
+}
+
+// The run of 4 cells at (x0, y), rows 16-byte aligned: reads, computes and
+// writes; returns the four tan^2.  The range tests of the eight divisions
+// and four reciprocal roots (see div_rn_by_rcp, rcp_sqrt_mid) are one: a
+// difference's magnitude lies in [2^-60, 2^60] or is zero (which, less one,
+// lies above every bound), a root's argument t2 + 1 is at least 1 or NaN.  A run
+// outside takes the general form cell by cell.  With a test and a branch for
+// each, the pass was bound by issue (8192^2 from uint16 with slope: 319 us).
+template <bool FROM_U16>
+__device__ __forceinline__ float4 normals_run(const NormalsArgs<FROM_U16>& a, const SpanDiv& d, int y, int x0)
+{
+    const int W = a.W, H = a.H;
+    const int64_t plane = (int64_t)W * H;
+    const int yl = y > 0 ? y - 1 : 0, yr = y < H - 1 ? y + 1 : H - 1;
+    const int64_t row = (int64_t)y * W;
+    const float4 c = a.h.at4(row + x0);
+    const float4 up = a.h.at4((int64_t)yl * W + x0);
+    const float4 dn = a.h.at4((int64_t)yr * W + x0);
+    const float left = x0 > 0 ? a.h.at(row + x0 - 1) : c.x;
+    const float right = x0 + 4 < W ? a.h.at(row + x0 + 4) : c.w;
+    if (FROM_U16) *reinterpret_cast<float4*>(a.h_out + row + x0) = c;
+    // differences and their spans: cells of the run's ends may be one-sided
+    // (or W == 1: not with W % 4 == 0); a single row has gy = 0
+    const float dx[4] = {__fsub_rn(c.y, left), __fsub_rn(c.z, c.x), __fsub_rn(c.w, c.y), __fsub_rn(right, c.z)};
+    const float dy[4] = {__fsub_rn(dn.x, up.x), __fsub_rn(dn.y, up.y), __fsub_rn(dn.z, up.z), __fsub_rn(dn.w, up.w)};
+    const bool one_l = x0 == 0, one_r = x0 + 4 >= W, one_y = yr - yl != 2;
+    const float dny = one_y ? d.den1 : d.den2, rdy = one_y ? d.rden1 : d.rden2;
+    float nx[4], ny[4], nz[4], t2[4];
+    uint32_t least = 0xffffffffu, most = 0u;
+    float top = 0.0f;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const bool one = k == 0 ? one_l : (k == 3 ? one_r : false);
+        const float den = one ? d.den1 : d.den2, rden = one ? d.rden1 : d.rden2;
+        const uint32_t bx = __float_as_uint(dx[k]) & 0x7fffffffu, by = __float_as_uint(dy[k]) & 0x7fffffffu;
+        least = min(least, min(bx - 1u, by - 1u));
+        most = max(most, max(bx, by));
+        const float gx = with_sign(div_rn_mid(dx[k], den, rden), dx[k]);
+        const float gy = with_sign(div_rn_mid(dy[k], dny, rdy), dy[k]);
+        t2[k] = __fadd_rn(__fmul_rn(gx, gx), __fmul_rn(gy, gy));
+        const float x = __fadd_rn(t2[k], 1.0f);
+        top = fmaxf(top, x);  // a NaN comes from a difference that is one, too
+        nz[k] = rcp_sqrt_mid(x);
+        nx[k] = __fmul_rn(-gx, nz[k]);
+        ny[k] = __fmul_rn(-gy, nz[k]);
+    }
+    const bool fast = least >= DIV_LOW - 1u && most <= DIV_HIGH && top <= 0x1p100f && d.den1 >= 0x1p-60f &&
+                      d.den2 <= 0x1p60f;
+    if (!fast) {
+#pragma unroll 1
+        for (int k = 0; k < 4; ++k) {
+            const bool one = k == 0 ? one_l : (k == 3 ? one_r : false);
+            const float gx = div_rn_by_rcp<true>(k == 0 ? dx[0] : (k == 1 ? dx[1] : (k == 2 ? dx[2] : dx[3])),
+                                                 one ? d.den1 : d.den2, one ? d.rden1 : d.rden2);
+            const float gy = yr > yl ? div_rn_by_rcp<true>(k == 0 ? dy[0] : (k == 1 ? dy[1] : (k == 2 ? dy[2] : dy[3])),
+                                                           dny, rdy)
+                                     : 0.0f;
+            float ox, oy, oz, ot;
+            normal_of(gx, gy, ox, oy, oz, ot);
+#pragma unroll
+            for (int m = 0; m < 4; ++m)
+                if (m == k) nx[m] = ox, ny[m] = oy, nz[m] = oz, t2[m] = ot;
+        }
+    }
+    if (a.nrm) {
+        *reinterpret_cast<float4*>(a.nrm + row + x0) = make_float4(nx[0], nx[1], nx[2], nx[3]);
+        *reinterpret_cast<float4*>(a.nrm + plane + row + x0) = make_float4(ny[0], ny[1], ny[2], ny[3]);
+        *reinterpret_cast<float4*>(a.nrm + 2 * plane + row + x0) = make_float4(nz[0], nz[1], nz[2], nz[3]);
+    }
+    const float4 t = make_float4(t2[0], t2[1], t2[2], t2[3]);
+    if (a.tan2) *reinterpret_cast<float4*>(a.tan2 + row + x0) = t;
+    if (a.slope_deg)
+        *reinterpret_cast<float4*>(a.slope_deg + row + x0) =
+            make_float4(slope_deg_of(t.x), slope_deg_of(t.y), slope_deg_of(t.z), slope_deg_of(t.w));
+    return t;
+}
+
+// The cells one by one: ragged rows and unaligned buffers.
+template <bool FROM_U16>
+__global__ void __launch_bounds__(256) k_normals(const __grid_constant__ NormalsArgs<FROM_U16> a)
+{
+    const int W = a.W, H = a.H;
     const int64_t plane = (int64_t)W * H;
     const uint32_t runs = (uint32_t)((W + 3) >> 2);
     const uint32_t items = runs * (uint32_t)H;
-    const float den1 = cs, den2 = __fmul_rn(cs, 2.0f);
-    const float rden1 = __frcp_rn(den1), rden2 = __frcp_rn(den2);  // the divisions: div_rn_by_rcp, = __fdiv_rn
+    const SpanDiv d = span_div(a.cs);
     for (uint32_t it = blockIdx.x * blockDim.x + threadIdx.x; it < items; it += gridDim.x * blockDim.x) {
         const int y = (int)(it / runs);
         const int x0 = (int)(it - (uint32_t)y * runs) * 4;
         const int yl = y > 0 ? y - 1 : 0, yr = y < H - 1 ? y + 1 : H - 1;
-        const float deny = yr - yl == 2 ? den2 : den1, rdeny = yr - yl == 2 ? rden2 : rden1;
+        const float deny = yr - yl == 2 ? d.den2 : d.den1, rdeny = yr - yl == 2 ? d.rden2 : d.rden1;
         const int64_t row = (int64_t)y * W;
-        if (vec4) {
-            const float4 c = h.at4(row + x0);
-            const float4 up = h.at4((int64_t)yl * W + x0);
-            const float4 dn = h.at4((int64_t)yr * W + x0);
-            const float left = x0 > 0 ? h.at(row + x0 - 1) : c.x;
-            const float right = x0 + 4 < W ? h.at(row + x0 + 4) : c.w;
-            if (FROM_U16) *reinterpret_cast<float4*>(h_out + row + x0) = c;
-            const float hc[6] = {left, c.x, c.y, c.z, c.w, right};
-            const float hu[4] = {up.x, up.y, up.z, up.w}, hd[4] = {dn.x, dn.y, dn.z, dn.w};
-            float o_nx[4], o_ny[4], o_nz[4], o_t2[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int x = x0 + k;
-                const int xl = x > 0 ? x - 1 : 0, xr = x < W - 1 ? x + 1 : W - 1;
-                float gx = 0.0f, gy = 0.0f;
-                const float h_r = x < W - 1 ? hc[k + 2] : hc[k + 1];
-                const float h_l = x > 0 ? hc[k] : hc[k + 1];
-                if (xr > xl)
-                    gx = xr - xl == 2 ? div_rn_by_rcp<true>(__fsub_rn(h_r, h_l), den2, rden2)
-                                      : div_rn_by_rcp<true>(__fsub_rn(h_r, h_l), den1, rden1);
-                if (yr > yl) gy = div_rn_by_rcp<true>(__fsub_rn(hd[k], hu[k]), deny, rdeny);
-                normal_of(gx, gy, o_nx[k], o_ny[k], o_nz[k], o_t2[k]);
+        const int x_end = x0 + 4 < W ? x0 + 4 : W;
+        for (int x = x0; x < x_end; ++x) {
+            const int xl = x > 0 ? x - 1 : 0, xr = x < W - 1 ? x + 1 : W - 1;
+            float gx = 0.0f, gy = 0.0f;
+            if (xr > xl)
+                gx = div_rn_by_rcp<true>(__fsub_rn(a.h.at(row + xr), a.h.at(row + xl)), xr - xl == 2 ? d.den2 : d.den1,
+                                         xr - xl == 2 ? d.rden2 : d.rden1);
+            if (yr > yl)
+                gy = div_rn_by_rcp<true>(__fsub_rn(a.h.at((int64_t)yr * W + x), a.h.at((int64_t)yl * W + x)), deny,
+                                         rdeny);
+            float nx, ny, nz, t2;
+            normal_of(gx, gy, nx, ny, nz, t2);
+            const int64_t i = row + x;
+            if (FROM_U16) a.h_out[i] = a.h.at(i);
+            if (a.nrm) {
+                a.nrm[i] = nx;
+                a.nrm[plane + i] = ny;
+                a.nrm[2 * plane + i] = nz;
             }
-            if (nrm) {
-                *reinterpret_cast<float4*>(nrm + row + x0) = make_float4(o_nx[0], o_nx[1], o_nx[2], o_nx[3]);
-                *reinterpret_cast<float4*>(nrm + plane + row + x0) = make_float4(o_ny[0], o_ny[1], o_ny[2], o_ny[3]);
-                *reinterpret_cast<float4*>(nrm + 2 * plane + row + x0) =
-                    make_float4(o_nz[0], o_nz[1], o_nz[2], o_nz[3]);
-            }
-            if (tan2) *reinterpret_cast<float4*>(tan2 + row + x0) = make_float4(o_t2[0], o_t2[1], o_t2[2], o_t2[3]);
-            if (slope_deg)
-                *reinterpret_cast<float4*>(slope_deg + row + x0) =
-                    make_float4(slope_deg_of(o_t2[0]), slope_deg_of(o_t2[1]), slope_deg_of(o_t2[2]),
-                                slope_deg_of(o_t2[3]));
-        } else {
-            const int x_end = x0 + 4 < W ? x0 + 4 : W;
-            for (int x = x0; x < x_end; ++x) {
-                const int xl = x > 0 ? x - 1 : 0, xr = x < W - 1 ? x + 1 : W - 1;
-                float gx = 0.0f, gy = 0.0f;
-                if (xr > xl)
-                    gx = div_rn_by_rcp<true>(__fsub_rn(h.at(row + xr), h.at(row + xl)), xr - xl == 2 ? den2 : den1,
-                                             xr - xl == 2 ? rden2 : rden1);
-                if (yr > yl)
-                    gy = div_rn_by_rcp<true>(__fsub_rn(h.at((int64_t)yr * W + x), h.at((int64_t)yl * W + x)), deny,
-                                             rdeny);
-                float nx, ny, nz, t2;
-                normal_of(gx, gy, nx, ny, nz, t2);
-                const int64_t i = row + x;
-                if (FROM_U16) h_out[i] = h.at(i);
-                if (nrm) {
-                    nrm[i] = nx;
-                    nrm[plane + i] = ny;
-                    nrm[2 * plane + i] = nz;
-                }
-                if (tan2) tan2[i] = t2;
-                if (slope_deg) slope_deg[i] = slope_deg_of(t2);
-            }
+            if (a.tan2) a.tan2[i] = t2;
+            if (a.slope_deg) a.slope_deg[i] = slope_deg_of(t2);
         }
     }
 }
@@ -228,6 +290,21 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int* total)
     *total = warp_sums[(blockDim.x >> 5) - 1];
     __syncthreads();
     return base + incl - v;
+}
+
+// Sum of v over the block, in thread 0 (call once per kernel: one barrier).
+__device__ __forceinline__ uint32_t block_total(int v)
+{
+    __shared__ int warp_total[RT_THREADS / 32];
+    const int t = __reduce_add_sync(0xffffffffu, v);
+    if ((threadIdx.x & 31) == 0) warp_total[threadIdx.x >> 5] = t;
+    __syncthreads();
+    int total = 0;
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int w = 0; w < RT_THREADS / 32; ++w) total += warp_total[w];
+    }
+    return (uint32_t)total;
 }
 
 // Selection bits of the RT_CELLS consecutive cells from `base` (bit k: cell
@@ -313,9 +390,49 @@ __global__ void __launch_bounds__(RT_THREADS) k_release_mask(const float* __rest
     const int64_t base = (int64_t)blockIdx.x * RT_TILE + (int64_t)threadIdx.x * RT_CELLS;
     const uint32_t bits = select_bits(tan2, base, n, t_lo, t_hi);
     if (mask) store_mask(mask, base, n, bits);
-    int total;
-    block_exclusive_scan(__popc(bits), &total);
-    if (threadIdx.x == 0) tile_count[blockIdx.x] = (uint32_t)total;
+    const uint32_t total = block_total(__popc(bits));
+    if (threadIdx.x == 0) tile_count[blockIdx.x] = total;
+}
+
+// Aligned rows (a run of 4 cells is 4 consecutive indices): a block makes the
+// normals of one release tile, and (tile_count not null) tests each tan^2
+// while it is in registers and writes the mask and the tile's count -- a1 and
+// the first release pass in one: tan^2 is not read back (4 of the 32 bytes
+// that the two passes move per cell) and a launch is saved.  Bound by HBM:
+// 8192^2 from uint16 with slope, normals and release 408 -> 313 us (86% of the
+// measured copy bandwidth).  A block per tile rather than a persistent
+// grid-stride loop, whose blocks all reached the same rows' end together.
+template <bool FROM_U16>
+__global__ void __launch_bounds__(RT_THREADS) k_normals_tiles(const __grid_constant__ NormalsArgs<FROM_U16> a,
+                                                                float t_lo, float t_hi, uint8_t* __restrict__ mask,
+                                                                uint32_t* __restrict__ tile_count)
+{
+    const uint32_t runs = (uint32_t)a.W >> 2, items = runs * (uint32_t)a.H;
+    const SpanDiv d = span_div(a.cs);
+    const uint32_t first = blockIdx.x * (uint32_t)(RT_TILE / 4);
+    const uint32_t y_first = first / runs, x_first = first - y_first * runs;  // in runs
+    int count = 0;
+#pragma unroll 1
+    for (uint32_t k = threadIdx.x; k < RT_TILE / 4; k += RT_THREADS) {
+        if (first + k >= items) break;
+        uint32_t y = y_first, x = x_first + k;
+        if (x >= runs) {
+            const uint32_t rows = x / runs;
+            y += rows;
+            x -= rows * runs;
+        }
+        const float4 t = normals_run<FROM_U16>(a, d, (int)y, (int)(4u * x));
+        if (!tile_count) continue;
+        const uint32_t sel = ((t_lo <= t.x && t.x <= t_hi) ? 1u : 0u) | ((t_lo <= t.y && t.y <= t_hi) ? 0x100u : 0u) |
+                             ((t_lo <= t.z && t.z <= t_hi) ? 0x10000u : 0u) |
+                             ((t_lo <= t.w && t.w <= t_hi) ? 0x1000000u : 0u);
+        if (mask) *reinterpret_cast<uint32_t*>(mask + 4 * (size_t)(first + k)) = sel;
+        count += __popc(sel);
+    }
+    if (tile_count) {
+        const uint32_t total = block_total(count);
+        if (threadIdx.x == 0) tile_count[blockIdx.x] = total;
+    }
 }
 
 // Exclusive scan of tile counts in one block of 1024 threads; also writes the
@@ -422,9 +539,8 @@ __global__ void __launch_bounds__(RT_THREADS) k_mask_count(const uint8_t* __rest
                                                            uint32_t* __restrict__ tile_count)
 {
     const int64_t base = (int64_t)blockIdx.x * RT_TILE + (int64_t)threadIdx.x * RT_CELLS;
-    int total;
-    block_exclusive_scan(__popc(mask_bits(mask, base, n)), &total);
-    if (threadIdx.x == 0) tile_count[blockIdx.x] = (uint32_t)total;
+    const uint32_t total = block_total(__popc(mask_bits(mask, base, n)));
+    if (threadIdx.x == 0) tile_count[blockIdx.x] = total;
 }
 
 // The scatter pass takes SC_RUNS consecutive runs per thread, so a block
@@ -546,11 +662,10 @@ __global__ void __launch_bounds__(RT_THREADS) k_release_texture_mask(const float
                                                                      uint32_t Wr, int64_t n, float scale,
                                                                      float t_lo, float t_hi,
                                                                      uint8_t* __restrict__ mask,
-                                                                     uint32_t* __restrict__ tile_count,
-                                                                     uint32_t tile0)
+                                                                     uint32_t* __restrict__ tile_count)
 {
     // the texture has fewer than 2^31 texels: 32-bit indices throughout
-    const uint32_t tile = tile0 + blockIdx.x;
+    const uint32_t tile = blockIdx.x;
     const uint32_t base = tile * (uint32_t)RT_TILE + threadIdx.x * (uint32_t)RT_CELLS;
     const uint32_t n32 = (uint32_t)n;
     const float wm1 = __int2float_rn(W - 1), hm1 = __int2float_rn(H - 1);
@@ -612,22 +727,23 @@ __global__ void __launch_bounds__(RT_THREADS) k_release_texture_mask(const float
         }
     }
     store_mask(mask, base, n, bits);
-    int total;
-    block_exclusive_scan(__popc(bits), &total);
-    if (threadIdx.x == 0) tile_count[tile] = (uint32_t)total;
+    const uint32_t total = block_total(__popc(bits));
+    if (threadIdx.x == 0) tile_count[tile] = total;
 }
 
 // Rows that share their tan^2 rows (R = 1, 2): texture rows b = 2^R j + 2^(R-1)
 // ... 2^R j + 2^(R-1) + 2^R - 1 all have their centres between DEM rows j and
 // j + 1, so their texels at one column interpolate the same two horizontal
 // interpolations, with their own vertical weights.  A block takes one tile
-// column (RT_TILE texels of a row; rows are whole tiles) of the 2^R rows of
-// group j = blockIdx.y, each thread a run of RT_CELLS texels in every row:
-// the tan^2 values and the horizontal interpolations are computed once for
-// the group, the vertical combination per row (the same operations, in the
-// same order, as k_release_texture_mask).  The 2^(R-1) rows above the first
-// group and below the last clamp their centres to the grid and take
-// k_release_texture_mask.
+// column (RT_TILE texels of a row; rows are whole tiles) of the rows of group
+// blockIdx.y, each thread a run of RT_CELLS texels in every row: the tan^2
+// values and the horizontal interpolations are computed once for the group,
+// the vertical combination per row (the same operations, in the same order, as
+// k_release_texture_mask).  Group 0 holds the 2^(R-1) rows above the first of
+// those and group H the 2^(R-1) below the last: their centres clamp to the
+// DEM's first and last row.  (Those rows in launches of their own, and a block
+// scan where only its total is wanted: 61 us for the mask of a 4096^2 DEM at
+// 2x.)
 template <int R, bool VEC>
 __global__ void __launch_bounds__(RT_THREADS) k_release_texture_rows(const float* __restrict__ tan2, int W, int H,
                                                                      uint32_t Wr, int64_t n, float scale,
@@ -636,20 +752,23 @@ __global__ void __launch_bounds__(RT_THREADS) k_release_texture_rows(const float
                                                                      uint32_t* __restrict__ tile_count)
 {
     using T = TexRun<R>;
-    constexpr int ROWS = 1 << R;
+    constexpr int ROWS = 1 << R, HALF = ROWS / 2;
     const uint32_t tiles_per_row = Wr / (uint32_t)RT_TILE;
-    const int j = (int)blockIdx.y;
-    const uint32_t b0 = (uint32_t)j * ROWS + (ROWS >> 1);  // first texture row of the group
+    const int group = (int)blockIdx.y;
+    const bool edge = group == 0 || group == H;
+    const int j = group == 0 ? 0 : group - 1;  // DEM row under the group
+    const int dj = j + 1 < H ? W : 0;          // to the row below, clamped
+    const uint32_t b0 = group == 0 ? 0u : (uint32_t)j * ROWS + HALF;  // first texture row of the group
     const uint32_t a = blockIdx.x * (uint32_t)RT_TILE + threadIdx.x * (uint32_t)RT_CELLS;
     const float hm1 = __int2float_rn(H - 1), wm1 = __int2float_rn(W - 1);
     float oy[ROWS], fy[ROWS];
 #pragma unroll
     for (int r = 0; r < ROWS; ++r) {
-        const float v = texel_centre(b0 + r, scale, hm1);  // in [j, j + 1): floor j, no clamp
+        const float v = texel_centre(b0 + r, scale, hm1);  // in [j, j + 1) (rows of the group)
         fy[r] = __fsub_rn(v, __int2float_rn(j));
         oy[r] = __fsub_rn(1.0f, fy[r]);
     }
-    const int row = j * W;  // dj = W: j + 1 <= H - 1
+    const int row = j * W;
     uint32_t bits[ROWS];
 #pragma unroll
     for (int r = 0; r < ROWS; ++r) bits[r] = 0u;
@@ -663,14 +782,14 @@ __global__ void __launch_bounds__(RT_THREADS) k_release_texture_rows(const float
             const bool whole = VEC && g >= T::DMIN && g + 3 <= T::DMAX + 1;
             if (whole && i == g) {
                 const float4 qt = __ldg(reinterpret_cast<const float4*>(p + i));
-                const float4 qb = __ldg(reinterpret_cast<const float4*>(p + W + i));
+                const float4 qb = __ldg(reinterpret_cast<const float4*>(p + dj + i));
                 top[i - T::DMIN] = qt.x, top[i - T::DMIN + 1] = qt.y, top[i - T::DMIN + 2] = qt.z,
                               top[i - T::DMIN + 3] = qt.w;
                 bot[i - T::DMIN] = qb.x, bot[i - T::DMIN + 1] = qb.y, bot[i - T::DMIN + 2] = qb.z,
                               bot[i - T::DMIN + 3] = qb.w;
             } else if (!whole) {
                 top[i - T::DMIN] = __ldg(p + i);
-                bot[i - T::DMIN] = __ldg(p + W + i);
+                bot[i - T::DMIN] = __ldg(p + dj + i);
             }
         }
 #pragma unroll
@@ -694,7 +813,7 @@ __global__ void __launch_bounds__(RT_THREADS) k_release_texture_rows(const float
             const float fx = __fsub_rn(u, __int2float_rn(i0));
             const int o = row + i0, di = i0 + 1 < W ? 1 : 0;
             const float t00 = __ldg(tan2 + o), t10 = __ldg(tan2 + o + di);
-            const float t01 = __ldg(tan2 + o + W), t11 = __ldg(tan2 + o + W + di);
+            const float t01 = __ldg(tan2 + o + dj), t11 = __ldg(tan2 + o + dj + di);
             const float ox = __fsub_rn(1.0f, fx);
             const float tp = __fadd_rn(__fmul_rn(t00, ox), __fmul_rn(t10, fx));
             const float bt = __fadd_rn(__fmul_rn(t01, ox), __fmul_rn(t11, fx));
@@ -705,12 +824,19 @@ __global__ void __launch_bounds__(RT_THREADS) k_release_texture_rows(const float
             }
         }
     }
+    __shared__ int s_count[ROWS][RT_THREADS / 32];
 #pragma unroll
     for (int r = 0; r < ROWS; ++r) {
-        store_mask(mask, (int64_t)(b0 + r) * Wr + a, n, bits[r]);
-        int total;
-        block_exclusive_scan(__popc(bits[r]), &total);
-        if (threadIdx.x == 0) tile_count[(b0 + r) * tiles_per_row + blockIdx.x] = (uint32_t)total;
+        if (!edge || r < HALF) store_mask(mask, (int64_t)(b0 + r) * Wr + a, n, bits[r]);
+        const int c = __reduce_add_sync(0xffffffffu, __popc(bits[r]));
+        if ((threadIdx.x & 31) == 0) s_count[r][threadIdx.x >> 5] = c;
+    }
+    __syncthreads();
+    if (threadIdx.x < (edge ? HALF : ROWS)) {
+        int total = 0;
+#pragma unroll
+        for (int w = 0; w < RT_THREADS / 32; ++w) total += s_count[threadIdx.x][w];
+        tile_count[(b0 + threadIdx.x) * tiles_per_row + blockIdx.x] = (uint32_t)total;
     }
 }
 
@@ -749,17 +875,35 @@ extern "C" awo_status awo_decode_u16(const uint16_t* d_q, awo_grid g, float scal
     return launch_status();
 }
 
+// Rows and buffers of a pass over runs of four cells are aligned for it.
+static bool runs_aligned(awo_grid g, const void* heights, size_t heights_align, const void* a, const void* b,
+                         const void* c, const void* d, const void* mask)
+{
+    const uintptr_t p = (uintptr_t)a | (uintptr_t)b | (uintptr_t)c | (uintptr_t)d;
+    return (g.width % 4) == 0 && ((uintptr_t)heights & (heights_align - 1)) == 0 && (p & 15u) == 0 &&
+           ((uintptr_t)mask & 3u) == 0;
+}
+
+template <bool FROM_U16>
+static awo_status launch_normals(const NormalsArgs<FROM_U16>& a, awo_grid g, bool aligned, cudaStream_t s)
+{
+    const int64_t n = cells_of(g);
+    if (aligned)
+        k_normals_tiles<FROM_U16><<<(unsigned)((n + RT_TILE - 1) / RT_TILE), RT_THREADS, 0, s>>>(a, 0.0f, 0.0f, nullptr,
+                                                                                                 nullptr);
+    else
+        k_normals<FROM_U16><<<stream_blocks((int64_t)((g.width + 3) / 4) * g.height, 256), 256, 0, s>>>(a);
+    return launch_status();
+}
+
 extern "C" awo_status awo_normals(const float* d_h, awo_grid g, float* d_normal, float* d_tan2,
                                   float* d_slope_deg, void* stream)
 {
     if (!d_h || !grid_ok(g)) return AWO_EINVAL;
     if (!d_normal && !d_tan2 && !d_slope_deg) return AWO_OK;
-    const int64_t items = (int64_t)((g.width + 3) / 4) * g.height;
-    auto a16 = [](const void* p) { return p == nullptr || (((uintptr_t)p) & 15u) == 0; };
-    const bool vec4 = (g.width % 4) == 0 && a16(d_h) && a16(d_normal) && a16(d_tan2) && a16(d_slope_deg);
-    k_normals<false><<<stream_blocks(items, 256), 256, 0, as_stream(stream)>>>(
-        HeightSrc<false>{d_h, 1.0f}, g.width, g.height, g.cell_size, d_normal, d_tan2, d_slope_deg, nullptr, vec4);
-    return launch_status();
+    return launch_normals(NormalsArgs<false>{{d_h, 1.0f}, g.width, g.height, g.cell_size, d_normal, d_tan2, d_slope_deg,
+                                             nullptr},
+                          g, runs_aligned(g, d_h, 16, d_normal, d_tan2, d_slope_deg, nullptr, nullptr), as_stream(stream));
 }
 
 extern "C" awo_status awo_normals_u16(const uint16_t* d_q, awo_grid g, float scale, float* d_h, float* d_normal,
@@ -767,13 +911,22 @@ extern "C" awo_status awo_normals_u16(const uint16_t* d_q, awo_grid g, float sca
 {
     if (!d_q || !d_h || !grid_ok(g) || !(scale > 0.0f) || !(scale < 3.0e38f)) return AWO_EINVAL;
     if (!d_normal && !d_tan2 && !d_slope_deg) return awo_decode_u16(d_q, g, scale, d_h, stream);
-    const int64_t items = (int64_t)((g.width + 3) / 4) * g.height;
-    auto a16 = [](const void* p) { return p == nullptr || (((uintptr_t)p) & 15u) == 0; };
-    const bool vec4 = (g.width % 4) == 0 && (((uintptr_t)d_q) & 7u) == 0 && a16(d_h) && a16(d_normal) &&
-                      a16(d_tan2) && a16(d_slope_deg);
-    k_normals<true><<<stream_blocks(items, 256), 256, 0, as_stream(stream)>>>(
-        HeightSrc<true>{d_q, scale}, g.width, g.height, g.cell_size, d_normal, d_tan2, d_slope_deg, d_h, vec4);
-    return launch_status();
+    return launch_normals(
+        NormalsArgs<true>{{d_q, scale}, g.width, g.height, g.cell_size, d_normal, d_tan2, d_slope_deg, d_h}, g,
+        runs_aligned(g, d_q, 8, d_normal, d_tan2, d_slope_deg, d_h, nullptr), as_stream(stream));
+}
+
+// The last two release passes: offsets of the tile counts, ordered scatter
+// from the mask (1 byte per cell instead of 4) or, without one, from tan^2.
+static void scan_and_scatter(const float* d_tan2, const uint8_t* d_mask, int64_t n, int tiles, float t_lo, float t_hi,
+                             const uint32_t* tile_count, uint32_t* tile_offset, uint32_t* d_cells, uint32_t* d_n,
+                             cudaStream_t s)
+{
+    k_release_scan<<<1, 1024, 0, s>>>(tile_count, tiles, tile_offset, d_n);
+    if (d_mask)
+        launch_mask_scatter(d_mask, n, tiles, tile_offset, d_cells, s);
+    else
+        k_release_scatter<<<tiles, RT_THREADS, 0, s>>>(d_tan2, n, t_lo, t_hi, tile_offset, d_cells);
 }
 
 extern "C" size_t awo_release_workspace_bytes(awo_grid g)
@@ -783,14 +936,22 @@ extern "C" size_t awo_release_workspace_bytes(awo_grid g)
     return (size_t)(2 * tiles * sizeof(uint32_t) + 256);
 }
 
+// The checks of awo_release on its arguments (the heights' are made by the caller).
+static awo_status release_args(const float* d_tan2, awo_grid g, double lo, double hi, const uint32_t* d_cells,
+                               const uint32_t* d_n, const void* d_ws, size_t ws_bytes)
+{
+    if (!d_tan2 || !d_cells || !d_n || !d_ws || !grid_ok(g)) return AWO_EINVAL;
+    if (!(lo >= 0.0) || !(hi < 90.0) || lo > hi) return AWO_EINVAL;
+    if ((((uintptr_t)d_ws) & 15u) != 0) return AWO_EINVAL;
+    return ws_bytes < awo_release_workspace_bytes(g) ? AWO_ENOMEM : AWO_OK;
+}
+
 extern "C" awo_status awo_release(const float* d_tan2, awo_grid g, double slope_lo_deg, double slope_hi_deg,
                                   uint8_t* d_mask, uint32_t* d_cells, uint32_t* d_n, void* d_ws, size_t ws_bytes,
                                   void* stream)
 {
-    if (!d_tan2 || !d_cells || !d_n || !d_ws || !grid_ok(g)) return AWO_EINVAL;
-    if (!(slope_lo_deg >= 0.0) || !(slope_hi_deg < 90.0) || slope_lo_deg > slope_hi_deg) return AWO_EINVAL;
-    if ((((uintptr_t)d_ws) & 15u) != 0) return AWO_EINVAL;
-    if (ws_bytes < awo_release_workspace_bytes(g)) return AWO_ENOMEM;
+    const awo_status st = release_args(d_tan2, g, slope_lo_deg, slope_hi_deg, d_cells, d_n, d_ws, ws_bytes);
+    if (st != AWO_OK) return st;
     const int64_t n = cells_of(g);
     const int tiles = (int)((n + RT_TILE - 1) / RT_TILE);
     uint32_t* tile_count = static_cast<uint32_t*>(d_ws);
@@ -798,12 +959,57 @@ extern "C" awo_status awo_release(const float* d_tan2, awo_grid g, double slope_
     const float t_lo = tan2_of_degrees(slope_lo_deg), t_hi = tan2_of_degrees(slope_hi_deg);
     cudaStream_t s = as_stream(stream);
     k_release_mask<<<tiles, RT_THREADS, 0, s>>>(d_tan2, n, t_lo, t_hi, d_mask, tile_count);
-    k_release_scan<<<1, 1024, 0, s>>>(tile_count, tiles, tile_offset, d_n);
-    if (d_mask)  // 1 byte per cell instead of 4
-        launch_mask_scatter(d_mask, n, tiles, tile_offset, d_cells, s);
-    else
-        k_release_scatter<<<tiles, RT_THREADS, 0, s>>>(d_tan2, n, t_lo, t_hi, tile_offset, d_cells);
+    scan_and_scatter(d_tan2, d_mask, n, tiles, t_lo, t_hi, tile_count, tile_offset, d_cells, d_n, s);
     return launch_status();
+}
+
+// a0 + a1 + b: the fused pass where rows are 16-byte aligned, else the calls
+// one after the other.
+template <bool FROM_U16>
+static awo_status normals_release(const NormalsArgs<FROM_U16>& a, awo_grid g, double lo, double hi, uint8_t* d_mask,
+                                  uint32_t* d_cells, uint32_t* d_n, void* d_ws, cudaStream_t s)
+{
+    const int64_t n = cells_of(g);
+    const int tiles = (int)((n + RT_TILE - 1) / RT_TILE);
+    uint32_t* tile_count = static_cast<uint32_t*>(d_ws);
+    const float t_lo = tan2_of_degrees(lo), t_hi = tan2_of_degrees(hi);
+    k_normals_tiles<FROM_U16><<<tiles, RT_THREADS, 0, s>>>(a, t_lo, t_hi, d_mask, tile_count);
+    scan_and_scatter(a.tan2, d_mask, n, tiles, t_lo, t_hi, tile_count, tile_count + tiles, d_cells, d_n, s);
+    return launch_status();
+}
+
+extern "C" awo_status awo_normals_release(const float* d_h, awo_grid g, float* d_normal, float* d_tan2,
+                                          float* d_slope_deg, double slope_lo_deg, double slope_hi_deg,
+                                          uint8_t* d_mask, uint32_t* d_cells, uint32_t* d_n, void* d_ws,
+                                          size_t ws_bytes, void* stream)
+{
+    if (!d_h) return AWO_EINVAL;
+    awo_status st = release_args(d_tan2, g, slope_lo_deg, slope_hi_deg, d_cells, d_n, d_ws, ws_bytes);
+    if (st != AWO_OK) return st;
+    if (runs_aligned(g, d_h, 16, d_normal, d_tan2, d_slope_deg, nullptr, d_mask))
+        return normals_release(
+            NormalsArgs<false>{{d_h, 1.0f}, g.width, g.height, g.cell_size, d_normal, d_tan2, d_slope_deg, nullptr}, g,
+            slope_lo_deg, slope_hi_deg, d_mask, d_cells, d_n, d_ws, as_stream(stream));
+    st = awo_normals(d_h, g, d_normal, d_tan2, d_slope_deg, stream);
+    return st != AWO_OK ? st
+                        : awo_release(d_tan2, g, slope_lo_deg, slope_hi_deg, d_mask, d_cells, d_n, d_ws, ws_bytes, stream);
+}
+
+extern "C" awo_status awo_normals_u16_release(const uint16_t* d_q, awo_grid g, float scale, float* d_h, float* d_normal,
+                                              float* d_tan2, float* d_slope_deg, double slope_lo_deg,
+                                              double slope_hi_deg, uint8_t* d_mask, uint32_t* d_cells, uint32_t* d_n,
+                                              void* d_ws, size_t ws_bytes, void* stream)
+{
+    if (!d_q || !d_h || !(scale > 0.0f) || !(scale < 3.0e38f)) return AWO_EINVAL;
+    awo_status st = release_args(d_tan2, g, slope_lo_deg, slope_hi_deg, d_cells, d_n, d_ws, ws_bytes);
+    if (st != AWO_OK) return st;
+    if (runs_aligned(g, d_q, 8, d_normal, d_tan2, d_slope_deg, d_h, d_mask))
+        return normals_release(
+            NormalsArgs<true>{{d_q, scale}, g.width, g.height, g.cell_size, d_normal, d_tan2, d_slope_deg, d_h}, g,
+            slope_lo_deg, slope_hi_deg, d_mask, d_cells, d_n, d_ws, as_stream(stream));
+    st = awo_normals_u16(d_q, g, scale, d_h, d_normal, d_tan2, d_slope_deg, stream);
+    return st != AWO_OK ? st
+                        : awo_release(d_tan2, g, slope_lo_deg, slope_hi_deg, d_mask, d_cells, d_n, d_ws, ws_bytes, stream);
 }
 
 // ---------------------------------------------------------------------------
@@ -858,11 +1064,7 @@ extern "C" awo_status awo_release_noalloc(const float* d_tan2, awo_grid g, doubl
     const float t_lo = tan2_of_degrees(slope_lo_deg), t_hi = tan2_of_degrees(slope_hi_deg);
     cudaStream_t s = as_stream(stream);
     k_release_mask<<<tiles, RT_THREADS, 0, s>>>(d_tan2, n, t_lo, t_hi, d_mask, tile_count);
-    k_release_scan<<<1, 1024, 0, s>>>(tile_count, tiles, tile_offset, d_n);
-    if (d_mask)  // 1 byte per cell instead of 4
-        launch_mask_scatter(d_mask, n, tiles, tile_offset, d_cells, s);
-    else
-        k_release_scatter<<<tiles, RT_THREADS, 0, s>>>(d_tan2, n, t_lo, t_hi, tile_offset, d_cells);
+    scan_and_scatter(d_tan2, d_mask, n, tiles, t_lo, t_hi, tile_count, tile_offset, d_cells, d_n, s);
     return launch_status();
 }
 
@@ -929,16 +1131,9 @@ extern "C" awo_status awo_release_texture(const float* d_tan2, awo_grid g, int32
                 : release_log2 == 2 ? (vec ? k_release_texture_mask<2, true> : k_release_texture_mask<2, false>)
                 : release_log2 == 3 ? k_release_texture_mask<3, false>
                                     : k_release_texture_mask<-1, false>;
-    if ((release_log2 == 1 || release_log2 == 2) && g.height >= 2 && wr % RT_TILE == 0) {
-        // rows are whole tiles: the row groups that share their tan^2 rows in
-        // one kernel, the 2^(r-1) clamped rows at each end in the other
-        const uint32_t tpr = (uint32_t)(wr / RT_TILE), edge = 1u << (release_log2 - 1);
-        const uint32_t last = edge + ((uint32_t)(g.height - 1) << release_log2);  // first bottom edge row
-        kern<<<edge * tpr, RT_THREADS, 0, s>>>(d_tan2, g.width, g.height, (uint32_t)wr, n, scale, t_lo, t_hi, d_mask,
-                                                tile_count, 0u);
-        kern<<<edge * tpr, RT_THREADS, 0, s>>>(d_tan2, g.width, g.height, (uint32_t)wr, n, scale, t_lo, t_hi, d_mask,
-                                                tile_count, last * tpr);
-        const dim3 grid(tpr, (unsigned)(g.height - 1));
+    if ((release_log2 == 1 || release_log2 == 2) && g.height >= 2 && g.height < 65535 && wr % RT_TILE == 0) {
+        // rows are whole tiles: one launch of row groups that share their tan^2 rows
+        const dim3 grid((unsigned)(wr / RT_TILE), (unsigned)g.height + 1u);  // at most 65535 groups
         if (release_log2 == 1) {
             if (vec)
                 k_release_texture_rows<1, true><<<grid, RT_THREADS, 0, s>>>(d_tan2, g.width, g.height, (uint32_t)wr,
@@ -956,7 +1151,7 @@ extern "C" awo_status awo_release_texture(const float* d_tan2, awo_grid g, int32
         }
     } else {
         kern<<<tiles, RT_THREADS, 0, s>>>(d_tan2, g.width, g.height, (uint32_t)wr, n, scale, t_lo, t_hi, d_mask,
-                                          tile_count, 0u);
+                                          tile_count);
     }
     k_release_scan<<<1, 1024, 0, s>>>(tile_count, tiles, tile_offset, d_n);
     launch_mask_scatter(d_mask, n, tiles, tile_offset, d_texels, s);

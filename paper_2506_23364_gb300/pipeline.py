@@ -13,9 +13,9 @@ import numpy as np
 import torch
 
 from . import (AWO_OK, Grid, SimParams, awo_finalize_lod, awo_normals, awo_normals_u16,
-               awo_release, awo_release_from_mask, awo_release_texture, awo_release_texture_dims,
+               awo_release_from_mask, awo_release_texture, awo_release_texture_dims,
                awo_release_texture_workspace_bytes, awo_release_workspace_bytes, awo_simulate,
-               awo_simulate_workspace_bytes, grid, lod_shapes, stats_dict)
+               awo_simulate_workspace_bytes, awo_terrain, grid, lod_shapes, stats_dict)
 
 SIM_CLEAR_OUTPUTS = 1
 
@@ -97,16 +97,17 @@ class Overlay:
     @_ranged("awo terrain")
     def terrain(self, slope_lo_deg: float, slope_hi_deg: float, decode_scale: float = 0.1, stream=None):
         """a0-b: decode, normals and release (the count stays on the device)."""
+        if not self.release_log2:  # decode, normals and selection in one pass
+            awo_terrain(self.q if self.quantised else self.h, self.g, decode_scale if self.quantised else None, self.h,
+                        self.normal, self.tan2, self.slope, slope_lo_deg, slope_hi_deg, self.mask, self.cells,
+                        self.n_rel, self.ws_rel, stream)
+            return
         if self.quantised:  # decode and normals in one pass
             awo_normals_u16(self.q, self.g, decode_scale, self.h, self.normal, self.tan2, self.slope, stream)
         else:
             awo_normals(self.h, self.g, self.normal, self.tan2, self.slope, stream)
-        if self.release_log2:
-            awo_release_texture(self.tan2, self.g, self.release_log2, slope_lo_deg, slope_hi_deg, self.mask,
-                                self.cells, self.n_rel, self.ws_rel, stream)
-        else:
-            awo_release(self.tan2, self.g, slope_lo_deg, slope_hi_deg, self.mask, self.cells, self.n_rel,
-                        self.ws_rel, stream)
+        awo_release_texture(self.tan2, self.g, self.release_log2, slope_lo_deg, slope_hi_deg, self.mask, self.cells,
+                            self.n_rel, self.ws_rel, stream)
 
     @_ranged("awo terrain (mask)")
     def terrain_from_mask(self, mask: torch.Tensor, decode_scale: float = 0.1, stream=None):
