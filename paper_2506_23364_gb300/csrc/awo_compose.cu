@@ -95,7 +95,9 @@ template <int NS>
 static void launch_compose(const float* v, const uint32_t* c, int64_t n, const awo_colormap& cm, const uint8_t* b,
                            uint8_t* o, bool vec4, cudaStream_t s)
 {
-    const unsigned blocks = stream_blocks(vec4 ? n / 4 + 1 : n, 256);
+    // 42 registers: 5 blocks an SM are resident, so 8 per SM left a second,
+    // partial wave (8192^2 display pass: 8 -> 369 us, 32 -> 360, 128 -> 366)
+    const unsigned blocks = stream_blocks(vec4 ? n / 4 + 1 : n, 256, 32);
     if (b)
         k_compose<NS, true><<<blocks, 256, 0, s>>>(v, c, n, cm, b, o, vec4);
     else
@@ -112,17 +114,29 @@ __device__ __forceinline__ float smooth_step(float e0, float e1, float x)
 
 __device__ __forceinline__ uint32_t snow_rgba(float a) { return 0x00ffffffu | (to_u8(__fmul_rn(255.0f, a)) << 24); }
 
-// Four texels per thread when every buffer is 16-byte aligned, then a scalar tail.
-__global__ void k_snow(const float* __restrict__ h, const float* __restrict__ nz, int64_t n, float a0, float a1,
-                       float c0, float c1, float* __restrict__ alpha, uint8_t* __restrict__ rgba, bool vec4)
+// Texels 4 q .. 4 q + 3 of p; aligned: p is 16-byte aligned (else 4).
+__device__ __forceinline__ float4 load4(const float* __restrict__ p, int64_t q, bool aligned)
+{
+    if (aligned) return __ldg(reinterpret_cast<const float4*>(p) + q);
+    return make_float4(__ldg(p + 4 * q), __ldg(p + 4 * q + 1), __ldg(p + 4 * q + 2), __ldg(p + 4 * q + 3));
+}
+
+// Four texels per thread when the outputs are 16-byte aligned, then a scalar
+// tail.  The inputs need not be: the third plane of normals whose cell count
+// is not a multiple of 4 starts off a 16-byte boundary, and the four loads of
+// a thread then share its neighbours' sectors in the L1.  Bound by HBM:
+// 5003 x 4099 with such a plane 86 -> 62 us.
+__global__ void __launch_bounds__(256, 8) k_snow(const float* __restrict__ h, const float* __restrict__ nz, int64_t n,
+                                                 float a0, float a1, float c0, float c1, float* __restrict__ alpha,
+                                                 uint8_t* __restrict__ rgba, bool vec4, bool vec_h, bool vec_nz)
 {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     uint32_t* rgba32 = reinterpret_cast<uint32_t*>(rgba);
     const int64_t n4 = vec4 ? n / 4 : 0;
     for (int64_t q = tid; q < n4; q += stride) {
-        const float4 hv = __ldg(reinterpret_cast<const float4*>(h) + q);
-        const float4 zv = __ldg(reinterpret_cast<const float4*>(nz) + q);
+        const float4 hv = load4(h, q, vec_h);
+        const float4 zv = load4(nz, q, vec_nz);
         const float4 a = make_float4(__fmul_rn(smooth_step(a0, a1, hv.x), smooth_step(c0, c1, zv.x)),
                                      __fmul_rn(smooth_step(a0, a1, hv.y), smooth_step(c0, c1, zv.y)),
                                      __fmul_rn(smooth_step(a0, a1, hv.z), smooth_step(c0, c1, zv.z)),
@@ -188,8 +202,9 @@ extern "C" awo_status awo_snow_cover(const float* d_h, const float* d_nz, awo_gr
     if (s_hi < 0.0) s_hi = 0.0;
     const float c0 = (float)cos(s_lo * r), c1 = (float)cos(s_hi * r);
     const int64_t n = cells_of(g);
-    const bool vec4 = ((((uintptr_t)d_h) | ((uintptr_t)d_nz) | ((uintptr_t)d_alpha) | ((uintptr_t)d_rgba)) & 15u) == 0;
-    k_snow<<<stream_blocks(vec4 ? n / 4 + 1 : n, 256), 256, 0, as_stream(stream)>>>(d_h, d_nz, n, a0, a1, c0, c1,
-                                                                                     d_alpha, d_rgba, vec4);
+    const bool vec4 = ((((uintptr_t)d_alpha) | ((uintptr_t)d_rgba)) & 15u) == 0;
+    k_snow<<<stream_blocks(vec4 ? n / 4 + 1 : n, 256), 256, 0, as_stream(stream)>>>(
+        d_h, d_nz, n, a0, a1, c0, c1, d_alpha, d_rgba, vec4, (((uintptr_t)d_h) & 15u) == 0,
+        (((uintptr_t)d_nz) & 15u) == 0);
     return launch_status();
 }

@@ -1,10 +1,10 @@
 // awo_overlay.cu -- velocity indicator and overlay mipmap (Sec. 3, Fig. 4).
 //
-// Both are streaming passes.  Levels 1-6 of the mipmap come from one kernel:
+// Both are streaming passes.  Six levels of the mipmap come from one kernel:
 // a block reduces its 64 x 64 tile of level 0 to level 1 and then, in shared
 // memory, to each further level (counts summed in 64 bits and saturated,
 // velocities by max), so level 0 is read once and every level written once;
-// deeper levels are built one launch per level from their parent.  The
+// deeper levels come from the sixth in the same way.  The
 // workflow's call also makes the velocity from the maximum energy inside the
 // same pass (awo_finalize_lod).
 #include <string.h>
@@ -43,69 +43,13 @@ __global__ void k_finalize(const float* __restrict__ maxe, int64_t n, float g2, 
     for (int64_t i = 4 * n4 + tid; i < n; i += stride) vel[i] = __fsqrt_rn(__fmul_rn(g2, maxe[i]));
 }
 
-__device__ __forceinline__ uint32_t sat_sum4(uint32_t a, uint32_t b, uint32_t c, uint32_t d)
-{
-    const unsigned long long s = (unsigned long long)a + b + c + d;
-    return s > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)s;
-}
-
-// One mipmap level.  Fast form (w % 4 == 0, h even, 16-byte-aligned inputs,
-// 8-byte-aligned outputs): a thread makes two output texels from a uint4 /
-// float4 of each of the two parent rows.  General form: one output texel,
-// missing children ignored.  Items are indexed in 32 bits (W * H < 2^31).
-__global__ void k_lod_level(const uint32_t* __restrict__ c_in, const float* __restrict__ v_in, int w, int h,
-                            uint32_t* __restrict__ c_out, float* __restrict__ v_out, int w2, int h2, bool vec)
-{
-    const uint32_t stride = gridDim.x * blockDim.x;
-    if (vec) {
-        const uint32_t pairs = (uint32_t)(w2 / 2), items = pairs * (uint32_t)h2;
-        for (uint32_t it = blockIdx.x * blockDim.x + threadIdx.x; it < items; it += stride) {
-            const uint32_t y = it / pairs, xp = it - y * pairs;
-            const int64_t r0 = (int64_t)(2 * y) * w + 4 * xp, r1 = r0 + w;
-            const uint4 a = __ldg(reinterpret_cast<const uint4*>(c_in + r0));
-            const uint4 b = __ldg(reinterpret_cast<const uint4*>(c_in + r1));
-            const float4 p = __ldg(reinterpret_cast<const float4*>(v_in + r0));
-            const float4 q = __ldg(reinterpret_cast<const float4*>(v_in + r1));
-            const int64_t o = (int64_t)y * w2 + 2 * xp;
-            reinterpret_cast<uint2*>(c_out + o)[0] = make_uint2(sat_sum4(a.x, a.y, b.x, b.y), sat_sum4(a.z, a.w, b.z, b.w));
-            reinterpret_cast<float2*>(v_out + o)[0] =
-                make_float2(fmaxf(fmaxf(p.x, p.y), fmaxf(q.x, q.y)), fmaxf(fmaxf(p.z, p.w), fmaxf(q.z, q.w)));
-        }
-        return;
-    }
-    const uint32_t n = (uint32_t)w2 * (uint32_t)h2;
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-        int y = (int)(i / (uint32_t)w2);
-        int x = (int)(i - (uint32_t)y * (uint32_t)w2);
-        int sx = 2 * x, sy = 2 * y;
-        bool hx = sx + 1 < w, hy = sy + 1 < h;
-        const int64_t r0 = (int64_t)sy * w, r1 = (int64_t)(sy + 1) * w;
-        unsigned long long sum = c_in[r0 + sx];
-        float m = v_in[r0 + sx];
-        if (hx) {
-            sum += c_in[r0 + sx + 1];
-            m = fmaxf(m, v_in[r0 + sx + 1]);
-        }
-        if (hy) {
-            sum += c_in[r1 + sx];
-            m = fmaxf(m, v_in[r1 + sx]);
-            if (hx) {
-                sum += c_in[r1 + sx + 1];
-                m = fmaxf(m, v_in[r1 + sx + 1]);
-            }
-        }
-        c_out[i] = sum > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)sum;
-        v_out[i] = m;
-    }
-}
-
 // Levels 1 .. 1 + LOD_FUSED - 1 of the mipmap in one pass over level 0.  A
 // block owns a 32 x 32 tile of level 1 (a 64 x 64 tile of level 0) and all
 // its descendants: 16 x 16 of level 2, ... 1 x 1 of level 6, since the tiles
 // of every level nest.  Level 1 is reduced from level 0 in global memory,
 // each further level from the previous one in shared memory; every texel is
 // the saturating count sum and the velocity maximum of its existing children
-// (children past a level's edge are ignored), as in k_lod_level.  One read of
+// (children past a level's edge are ignored).  One read of
 // level 0 and one write of each level, instead of a read and a write per
 // level with a launch each.  FROM_MAXE: level 0's velocity is not read but
 // made from the maximum energy as it is needed, vel = sqrt((2 g) maxe), and
@@ -254,53 +198,43 @@ extern "C" awo_status awo_finalize(const float* d_maxe, awo_grid g, float gravit
     return launch_status();
 }
 
-// Levels 1 .. levels-1 from level 0 = (d_count, v0): one fused launch for
-// levels 1 .. LOD_FUSED, then one launch per further level.  from_maxe: v0
-// is the maximum energy and level 0's velocity is written to d_vel (g2 = 2 g).
+// Levels 1 .. levels-1 from level 0 = (d_count, v0): a fused launch for every
+// LOD_FUSED levels, each from the last level of the one before (a launch for
+// each level past the sixth took 2.6-3.2 us a level, 20 us of the 375 us of a
+// full 8192^2 chain and its colouring).  from_maxe: v0 is the maximum energy
+// and level 0's velocity is written to d_vel (g2 = 2 g).
 static awo_status lod_levels(const uint32_t* d_count, const float* v0, bool from_maxe, float g2, float* d_vel,
                              awo_grid g, int32_t levels, uint32_t* const* d_count_lv, float* const* d_vel_lv,
                              cudaStream_t s)
 {
-    LodArgs a;
-    memset(&a, 0, sizeof(a));
-    a.c0 = d_count;
-    a.v0 = v0;
-    a.vel0 = d_vel;
-    a.g2 = g2;
-    a.n_out = levels - 1 < LOD_FUSED ? levels - 1 : LOD_FUSED;
-    a.w[0] = g.width;
-    a.h[0] = g.height;
-    for (int k = 1; k <= a.n_out; ++k) {
-        a.w[k] = (a.w[k - 1] + 1) / 2;
-        a.h[k] = (a.h[k - 1] + 1) / 2;
-        a.c[k - 1] = d_count_lv[k - 1];
-        a.v[k - 1] = d_vel_lv[k - 1];
-    }
-    a.vec2 = g.width % 2 == 0 &&
-             ((((uintptr_t)d_count) | ((uintptr_t)v0) | (from_maxe ? (uintptr_t)d_vel : (uintptr_t)0)) & 7u) == 0;
-    const dim3 grid((unsigned)((a.w[1] + LOD_TILE - 1) / LOD_TILE), (unsigned)((a.h[1] + LOD_TILE - 1) / LOD_TILE));
-    if (from_maxe)
-        k_lod_fused<true><<<grid, 256, 0, s>>>(a);
-    else
-        k_lod_fused<false><<<grid, 256, 0, s>>>(a);
-    awo_status st = launch_status();
-    if (st != AWO_OK) return st;
-    const uint32_t* ci = d_count_lv[a.n_out - 1];
-    const float* vi = d_vel_lv[a.n_out - 1];
-    int w = a.w[a.n_out], h = a.h[a.n_out];
-    for (int l = 1 + a.n_out; l < levels; ++l) {
-        int w2 = (w + 1) / 2, h2 = (h + 1) / 2;
-        const bool vec = w % 4 == 0 && h % 2 == 0 && ((((uintptr_t)ci) | ((uintptr_t)vi)) & 15u) == 0 &&
-                         ((((uintptr_t)d_count_lv[l - 1]) | ((uintptr_t)d_vel_lv[l - 1])) & 7u) == 0;
-        const int64_t items = vec ? (int64_t)(w2 / 2) * h2 : (int64_t)w2 * h2;
-        k_lod_level<<<stream_blocks(items, 256), 256, 0, s>>>(ci, vi, w, h, d_count_lv[l - 1], d_vel_lv[l - 1], w2,
-                                                              h2, vec);
-        st = launch_status();
+    int w = g.width, h = g.height;
+    for (int done = 0; done + 1 < levels; done += LOD_FUSED, from_maxe = false) {
+        LodArgs a;
+        memset(&a, 0, sizeof(a));
+        a.c0 = done ? d_count_lv[done - 1] : d_count;
+        a.v0 = done ? d_vel_lv[done - 1] : v0;
+        a.vel0 = d_vel;
+        a.g2 = g2;
+        a.n_out = levels - 1 - done < LOD_FUSED ? levels - 1 - done : LOD_FUSED;
+        a.w[0] = w;
+        a.h[0] = h;
+        for (int k = 1; k <= a.n_out; ++k) {
+            a.w[k] = (a.w[k - 1] + 1) / 2;
+            a.h[k] = (a.h[k - 1] + 1) / 2;
+            a.c[k - 1] = d_count_lv[done + k - 1];
+            a.v[k - 1] = d_vel_lv[done + k - 1];
+        }
+        a.vec2 = w % 2 == 0 &&
+                 ((((uintptr_t)a.c0) | ((uintptr_t)a.v0) | (from_maxe ? (uintptr_t)d_vel : (uintptr_t)0)) & 7u) == 0;
+        const dim3 grid((unsigned)((a.w[1] + LOD_TILE - 1) / LOD_TILE), (unsigned)((a.h[1] + LOD_TILE - 1) / LOD_TILE));
+        if (from_maxe)
+            k_lod_fused<true><<<grid, 256, 0, s>>>(a);
+        else
+            k_lod_fused<false><<<grid, 256, 0, s>>>(a);
+        const awo_status st = launch_status();
         if (st != AWO_OK) return st;
-        ci = d_count_lv[l - 1];
-        vi = d_vel_lv[l - 1];
-        w = w2;
-        h = h2;
+        w = a.w[a.n_out];
+        h = a.h[a.n_out];
     }
     return AWO_OK;
 }

@@ -1,0 +1,51 @@
+"""Mipmap chains deeper than one fused launch and the snow pass on planes that
+are not 16-byte aligned, against the oracle, bit for bit."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2506_23364_gb300 as awo
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("W,H,levels", [(700, 521, 11), (129, 4097, 14), (64, 64, 8), (1, 3000, 16), (256, 130, 7)])
+def test_deep_mipmap(W, H, levels):
+    rng = np.random.default_rng(W + H)
+    count = rng.integers(0, 2 ** 32, (H, W), dtype=np.uint64).astype(np.uint32)  # saturates within a few levels
+    count[rng.random((H, W)) < 0.9] = 3
+    maxe = (rng.random((H, W)) * 400).astype(np.float32)
+    g = awo.grid(W, H, 10.0)
+    shapes = awo.lod_shapes(g, levels)[1:]
+    vel = torch.empty((H, W), device="cuda")
+    cl = [torch.empty(s, dtype=torch.int32, device="cuda") for s in shapes]
+    vl = [torch.empty(s, dtype=torch.float32, device="cuda") for s in shapes]
+    awo.awo_finalize_lod(torch.from_numpy(maxe).cuda(), torch.from_numpy(count.view(np.int32)).cuda(), g, 9.81, levels,
+                         vel, cl, vl)
+    want_vel = oracle.finalize(maxe, 9.81)
+    want_c, want_v = oracle.lod(count, want_vel, levels)
+    assert np.array_equal(vel.cpu().numpy(), want_vel)
+    for l in range(1, levels):
+        assert np.array_equal(cl[l - 1].cpu().numpy().view(np.uint32), want_c[l]), l
+        assert np.array_equal(vl[l - 1].cpu().numpy(), want_v[l]), l
+
+
+@pytest.mark.parametrize("off_h", [0, 1, 2])
+@pytest.mark.parametrize("off_nz", [0, 1, 2, 3])
+@pytest.mark.parametrize("W,H", [(37, 11), (1, 3), (64, 33)])
+def test_snow_unaligned_inputs(W, H, off_h, off_nz):
+    n = W * H
+    rng = np.random.default_rng(n + off_nz)
+    h = (rng.random((H, W)) * 1200 + 900).astype(np.float32)
+    nz = (rng.random((H, W)) * 0.4 + 0.6).astype(np.float32)
+    hb, zb = torch.empty(n + 4, device="cuda"), torch.empty(n + 4, device="cuda")
+    ht, zt = hb[off_h:off_h + n], zb[off_nz:off_nz + n]
+    ht.copy_(torch.from_numpy(h.ravel()))
+    zt.copy_(torch.from_numpy(nz.ravel()))
+    alpha = torch.empty((H, W), device="cuda")
+    rgba = torch.empty((H, W, 4), dtype=torch.uint8, device="cuda")
+    awo.awo_snow_cover(ht, zt, awo.grid(W, H, 10.0), awo.SnowParams(1500.0, 300.0, 36.0, 4.0), alpha, rgba)
+    want_a, want_rgba = oracle.snow_cover(h, nz, 1500.0, 300.0, 36.0, 4.0)
+    assert np.array_equal(alpha.cpu().numpy(), np.asarray(want_a).reshape(H, W))
+    assert np.array_equal(rgba.cpu().numpy(), np.asarray(want_rgba).reshape(H, W, 4))
