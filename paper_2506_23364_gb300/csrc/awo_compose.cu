@@ -95,9 +95,14 @@ template <int NS>
 static void launch_compose(const float* v, const uint32_t* c, int64_t n, const awo_colormap& cm, const uint8_t* b,
                            uint8_t* o, bool vec4, cudaStream_t s)
 {
-    // 42 registers: 5 blocks an SM are resident, so 8 per SM left a second,
-    // partial wave (8192^2 display pass: 8 -> 369 us, 32 -> 360, 128 -> 366)
-    const unsigned blocks = stream_blocks(vec4 ? n / 4 + 1 : n, 256, 32);
+    // 42 registers: 5 blocks an SM are resident, so a grid of 8 per SM leaves a
+    // second, partial wave (8192^2 display pass: 8 -> 369 us, 32 -> 360, 128 ->
+    // 366); but each thread should have four groups or more (1984 x 2496: 34.8 us
+    // with four, 36.1 with one)
+    const int64_t groups = vec4 ? n / 4 + 1 : n;
+    const unsigned blocks = stream_blocks(groups, 256, groups >= (int64_t)sm_count() * 32 * 256 * 4
+                                                           ? 32
+                                                           : (groups >= (int64_t)sm_count() * 16 * 256 * 4 ? 16 : 8));
     if (b)
         k_compose<NS, true><<<blocks, 256, 0, s>>>(v, c, n, cm, b, o, vec4);
     else
@@ -126,6 +131,7 @@ __device__ __forceinline__ float4 load4(const float* __restrict__ p, int64_t q, 
 // is not a multiple of 4 starts off a 16-byte boundary, and the four loads of
 // a thread then share its neighbours' sectors in the L1.  Bound by HBM:
 // 5003 x 4099 with such a plane 86 -> 62 us.
+template <bool ALIGNED>
 __global__ void __launch_bounds__(256, 8) k_snow(const float* __restrict__ h, const float* __restrict__ nz, int64_t n,
                                                  float a0, float a1, float c0, float c1, float* __restrict__ alpha,
                                                  uint8_t* __restrict__ rgba, bool vec4, bool vec_h, bool vec_nz)
@@ -135,8 +141,8 @@ __global__ void __launch_bounds__(256, 8) k_snow(const float* __restrict__ h, co
     uint32_t* rgba32 = reinterpret_cast<uint32_t*>(rgba);
     const int64_t n4 = vec4 ? n / 4 : 0;
     for (int64_t q = tid; q < n4; q += stride) {
-        const float4 hv = load4(h, q, vec_h);
-        const float4 zv = load4(nz, q, vec_nz);
+        const float4 hv = load4(h, q, ALIGNED || vec_h);
+        const float4 zv = load4(nz, q, ALIGNED || vec_nz);
         const float4 a = make_float4(__fmul_rn(smooth_step(a0, a1, hv.x), smooth_step(c0, c1, zv.x)),
                                      __fmul_rn(smooth_step(a0, a1, hv.y), smooth_step(c0, c1, zv.y)),
                                      __fmul_rn(smooth_step(a0, a1, hv.z), smooth_step(c0, c1, zv.z)),
@@ -203,8 +209,9 @@ extern "C" awo_status awo_snow_cover(const float* d_h, const float* d_nz, awo_gr
     const float c0 = (float)cos(s_lo * r), c1 = (float)cos(s_hi * r);
     const int64_t n = cells_of(g);
     const bool vec4 = ((((uintptr_t)d_alpha) | ((uintptr_t)d_rgba)) & 15u) == 0;
-    k_snow<<<stream_blocks(vec4 ? n / 4 + 1 : n, 256), 256, 0, as_stream(stream)>>>(
-        d_h, d_nz, n, a0, a1, c0, c1, d_alpha, d_rgba, vec4, (((uintptr_t)d_h) & 15u) == 0,
-        (((uintptr_t)d_nz) & 15u) == 0);
+    const bool vec_h = (((uintptr_t)d_h) & 15u) == 0, vec_nz = (((uintptr_t)d_nz) & 15u) == 0;
+    auto kern = vec_h && vec_nz ? k_snow<true> : k_snow<false>;
+    kern<<<stream_blocks(vec4 ? n / 4 + 1 : n, 256), 256, 0, as_stream(stream)>>>(d_h, d_nz, n, a0, a1, c0, c1, d_alpha,
+                                                                                  d_rgba, vec4, vec_h, vec_nz);
     return launch_status();
 }
