@@ -30,7 +30,7 @@ namespace awo {
 struct SoftArgs {
     const float* h;
     int W, H;
-    float Wm1, Hm1, P, oneP, R, s;
+    float Wm1, Hm1, P, oneP, R, R23, s;  // (as in SimArgs)
     float kD, muD, D;      // drag_k*D, mu*D, D = s*cell_size (metres)
     float mu, k;           // for the log-parameter chain rule
     float inv_tau;
@@ -67,7 +67,8 @@ __global__ void __launch_bounds__(256) k_soft_starts(const __grid_constant__ Sof
     const uint32_t n_cells = soft_count(a);
     unsigned long long bad = 0ull;
     for (uint32_t ci = blockIdx.x * blockDim.x + threadIdx.x; ci < n_cells; ci += gridDim.x * blockDim.x) {
-        const CellStart st = cell_start(a.h, a.W, a.H, a.n_grid, __ldg(a.cells + ci));
+        CellStart st = cell_start(a.h, a.W, a.H, a.n_grid, __ldg(a.cells + ci));
+        first_vector(st, a.P, a.oneP);
         a.starts[ci] = st;
         bad += st.xy == ~0u ? 1ull : 0ull;
     }
@@ -91,14 +92,21 @@ constexpr uint32_t SOFT_REFILL_IDLE = 4;
 // 0-1 and 2-3 of block n >> 1; lanes start at n = 0 and move in pairs).  Per
 // particle the arithmetic is that of the hard mode's moves plus the
 // survival, its tangents and the deposits, in a fixed order.
+// Bound by issue (forward 80% of issue slots, L2 26%).  1024^2, 128 particles
+// per cell, 83 M moves: forward 732 -> 694 us, backward 902 -> 783 us against
+// a branch per way to end and per normalisation and the footprint (6
+// registers) kept as state; the backward's 64 registers instead of 66 (8
+// blocks an SM instead of 7, an 8-byte spill) are 821 -> 788 of that.
 template <bool GRAD, bool TEX>
-__global__ void __launch_bounds__(SOFT_THREADS) k_soft(const __grid_constant__ SoftArgs a)
+__global__ void __launch_bounds__(SOFT_THREADS, GRAD ? 8 : 9) k_soft(const __grid_constant__ SoftArgs a)
 {
     const int lane = threadIdx.x & 31;
     const unsigned lane_lt = (1u << lane) - 1u;
     const uint32_t n_cells = soft_count(a);
     const unsigned long long total = (unsigned long long)n_cells * a.N;
     const unsigned long long warps = (unsigned long long)gridDim.x * (blockDim.x >> 5);
+    // a few particles: fewer warps a block, so that they spread over the SMs
+    if (total <= 32ull * gridDim.x * (threadIdx.x >> 5)) return;
     unsigned long long chunk = total / (warps * SOFT_CHUNKS_PER_WARP);
     chunk = chunk < 32ull ? 32ull : (chunk > SOFT_CHUNK_MAX ? (unsigned long long)SOFT_CHUNK_MAX : chunk);
     chunk &= ~31ull;
@@ -110,7 +118,7 @@ __global__ void __launch_bounds__(SOFT_THREADS) k_soft(const __grid_constant__ S
     bool live = false;
     uint32_t ci = 0u, cell = 0u, j = 0u, n = 0u, last = 0u;
     float u = 0.f, v = 0.f, z = 0.f, dx = 0.f, dy = 0.f, e = 0.f, S = 1.f, w = 0.f;
-    float fx = 0.f, fy = 0.f, h00 = 0.f, h10 = 0.f, h01 = 0.f, h11 = 0.f;
+    float sga = 0.f, sgb = 0.f;  // gradient of the patch at the position (AWO_LANE_STATE)
     long long Q = 0;  // forward: cumulative fixed-point deposit
     float tmu = 0.f, tk = 0.f, smu = 0.f, sk = 0.f, acc_mu = 0.f, acc_k = 0.f, acc_w = 0.f;  // backward
     // the lane's counters
@@ -147,83 +155,73 @@ __global__ void __launch_bounds__(SOFT_THREADS) k_soft(const __grid_constant__ S
         }
     };
 
-    // One move of a live lane's particle with random words WX, WY (the move
-    // loop of the hard mode: a particle ends at max_steps moves, with no
-    // direction, outside the grid, or when S < 1e-7 after a move).
-    auto move = [&](uint32_t WX, uint32_t WY) {
-        if (!live) return;
-        if (n >= a.max_steps) {
-            finish();
-            return;
-        }
-        const float ox = __fsub_rn(1.0f, fx), oy = __fsub_rn(1.0f, fy);
-        const float ga = __fadd_rn(__fmul_rn(__fsub_rn(h10, h00), oy), __fmul_rn(__fsub_rn(h11, h01), fy));
-        const float gb = __fadd_rn(__fmul_rn(__fsub_rn(h01, h00), ox), __fmul_rn(__fsub_rn(h11, h10), fx));
-        const float gn2 = __fadd_rn(__fmul_rn(ga, ga), __fmul_rn(gb, gb));
-        float gx = dx, gy = dy;
-        if (n != 0u && gn2 != 0.0f) {
-            const float ginv = rcp_sqrt_rn(gn2);
-            gx = __fmul_rn(-ga, ginv);
-            gy = __fmul_rn(-gb, ginv);
-        }
-        const float xix = uniform_pm1(WX);
-        const float xiy = uniform_pm1(WY);
-        const float rx = __fadd_rn(__fadd_rn(__fmul_rn(a.P, dx), __fmul_rn(a.oneP, gx)), __fmul_rn(a.R, xix));
-        const float ry = __fadd_rn(__fadd_rn(__fmul_rn(a.P, dy), __fmul_rn(a.oneP, gy)), __fmul_rn(a.R, xiy));
+    // One move of the particle in every lane, live or not, with random words
+    // WX, WY (FIRST: it may be the particle's first).  The direction, step and
+    // footprint are those of the hard mode (AWO_MOVE_WORDS), without branches;
+    // then the lanes that move take their energy, survival and deposit, and
+    // the others end: at max_steps moves, with no direction, outside the
+    // grid, or when S < 1e-7 after a move.
+    auto move = [&](bool may_be_first, uint32_t WX, uint32_t WY) {
+        const bool first = may_be_first && n == 0u;
+        const float gn2 = __fadd_rn(__fmul_rn(sga, sga), __fmul_rn(sgb, sgb));
+        const float ginv = rcp_sqrt_mid(gn2);
+        const float mx = __fadd_rn(__fmul_rn(a.P, dx), __fmul_rn(a.oneP, __fmul_rn(-sga, ginv)));
+        const float my = __fadd_rn(__fmul_rn(a.P, dy), __fmul_rn(a.oneP, __fmul_rn(-sgb, ginv)));
+        const float rx = __fadd_rn(first ? dx : mx, __fmaf_rn(a.R23, __uint2float_rn(WX >> 8), -a.R));
+        const float ry = __fadd_rn(first ? dy : my, __fmaf_rn(a.R23, __uint2float_rn(WY >> 8), -a.R));
         const float r2 = __fadd_rn(__fmul_rn(rx, rx), __fmul_rn(ry, ry));
-        if (r2 == 0.0f) {
-            finish();
-            return;
-        }
-        const float rinv = rcp_sqrt_rn(r2);
-        dx = __fmul_rn(rx, rinv);
-        dy = __fmul_rn(ry, rinv);
-        const float u1 = __fadd_rn(u, __fmul_rn(a.s, dx));
-        const float v1 = __fadd_rn(v, __fmul_rn(a.s, dy));
-        if (!(u1 >= 0.0f && u1 <= a.Wm1 && v1 >= 0.0f && v1 <= a.Hm1)) {
-            finish();
-            return;
-        }
+        const float rinv = rcp_sqrt_mid(r2);
+        float ndx = __fmul_rn(rx, rinv), ndy = __fmul_rn(ry, rinv);
+        const uint32_t chk = max(first ? 0u : mid_offset(gn2), mid_offset(r2));
+        if (__any_sync(0xffffffffu, live && chk > MID_SPAN))
+            general_direction(first, sga, sgb, dx, dy, a.P, a.oneP, a.R, WX, WY, ndx, ndy);
+        const float u1 = __fadd_rn(u, __fmul_rn(a.s, ndx));
+        const float v1 = __fadd_rn(v, __fmul_rn(a.s, ndy));
+        // as unsigned compares of the bits: see AWO_MOVE_WORDS
+        const bool go = live && n < a.max_steps && __float_as_uint(u1) <= __float_as_uint(a.Wm1) &&
+                        __float_as_uint(v1) <= __float_as_uint(a.Hm1);
         const Foot f = foot_at<TEX ? 1 : 0>(a, u1, v1);
-        const float z1 = bilinear(f, __fsub_rn(1.0f, f.fx), __fsub_rn(1.0f, f.fy));
-        const float e1 = __fsub_rn(__fadd_rn(__fsub_rn(e, __fmul_rn(a.kD, e)), __fsub_rn(z, z1)), a.muD);
-        const float sig = 1.0f / (1.0f + expf(-e1 * a.inv_tau));
-        const float S1 = S * sig;
-        const uint32_t c1 = (uint32_t)(f.j0 + (f.fy >= 0.5f ? 1 : 0)) * (uint32_t)a.W +
-                            (uint32_t)(f.i0 + (f.fx >= 0.5f ? 1 : 0));
-        if (GRAD) {
-            const float tmu1 = (1.0f - a.kD) * tmu - a.D;
-            const float tk1 = (1.0f - a.kD) * tk - a.D * e;
-            const float ds = sig * (1.0f - sig) * a.inv_tau;
-            const float smu1 = smu * sig + S * ds * tmu1;
-            const float sk1 = sk * sig + S * ds * tk1;
-            const float G = __ldg(a.grad + c1);
-            acc_mu += G * (smu - smu1);
-            acc_k += G * (sk - sk1);
-            acc_w += G * (S - S1);
-            tmu = tmu1;
-            tk = tk1;
-            smu = smu1;
-            sk = sk1;
-        } else {
-            const long long Q1 = __float2ll_rn((1.0f - S1) * w * FIX_SCALE);
-            if (Q1 != Q) atomicAdd(a.deposit + c1, (unsigned long long)(Q1 - Q));
-            Q = Q1;
+        const float fox = __fsub_rn(1.0f, f.fx), foy = __fsub_rn(1.0f, f.fy);
+        const float z1 = bilinear(f, fox, foy);
+        bool ends = live && !go;
+        if (go) {
+            const float e1 = __fsub_rn(__fadd_rn(__fsub_rn(e, __fmul_rn(a.kD, e)), __fsub_rn(z, z1)), a.muD);
+            const float sig = 1.0f / (1.0f + expf(-e1 * a.inv_tau));
+            const float S1 = S * sig;
+            const uint32_t c1 = (uint32_t)visit_axis(v1) * (uint32_t)a.W + (uint32_t)visit_axis(u1);
+            if (GRAD) {
+                const float tmu1 = (1.0f - a.kD) * tmu - a.D;
+                const float tk1 = (1.0f - a.kD) * tk - a.D * e;
+                const float ds = sig * (1.0f - sig) * a.inv_tau;
+                const float smu1 = smu * sig + S * ds * tmu1;
+                const float sk1 = sk * sig + S * ds * tk1;
+                const float G = __ldg(a.grad + c1);
+                acc_mu += G * (smu - smu1);
+                acc_k += G * (sk - sk1);
+                acc_w += G * (S - S1);
+                tmu = tmu1;
+                tk = tk1;
+                smu = smu1;
+                sk = sk1;
+            } else {
+                const long long Q1 = __float2ll_rn((1.0f - S1) * w * FIX_SCALE);
+                if (Q1 != Q) atomicAdd(a.deposit + c1, (unsigned long long)(Q1 - Q));
+                Q = Q1;
+            }
+            u = u1;
+            v = v1;
+            e = e1;
+            S = S1;
+            last = c1;
+            ++n;
+            ends = S1 < SOFT_S_MIN;
         }
-        u = u1;
-        v = v1;
         z = z1;
-        e = e1;
-        S = S1;
-        fx = f.fx;
-        fy = f.fy;
-        h00 = f.h00;
-        h10 = f.h10;
-        h01 = f.h01;
-        h11 = f.h11;
-        last = c1;
-        ++n;
-        if (S1 < SOFT_S_MIN) finish();
+        dx = ndx;
+        dy = ndy;
+        sga = __fadd_rn(__fmul_rn(__fsub_rn(f.h10, f.h00), foy), __fmul_rn(__fsub_rn(f.h11, f.h01), f.fy));
+        sgb = __fadd_rn(__fmul_rn(__fsub_rn(f.h01, f.h00), fox), __fmul_rn(__fsub_rn(f.h11, f.h10), f.fx));
+        if (ends) finish();
     };
 
     while (true) {
@@ -273,7 +271,7 @@ __global__ void __launch_bounds__(SOFT_THREADS) k_soft(const __grid_constant__ S
                     e = 0.f;
                     S = 1.f;
                     w = __ldg(a.weight + c);
-                    fx = fy = h00 = h10 = h01 = h11 = 0.f;
+                    sga = sgb = 0.f;
                     Q = 0;
                     tmu = tk = smu = sk = acc_mu = acc_k = acc_w = 0.f;
                     ++traj;
@@ -288,8 +286,8 @@ __global__ void __launch_bounds__(SOFT_THREADS) k_soft(const __grid_constant__ S
         }
         // moves n and n + 1 from one Philox block: every live lane is at an even n
         const uint4 r = philox4x32_10(make_uint4(cell, j, n >> 1, 0u), a.keys);
-        move(r.x, r.y);
-        move(r.z, r.w);
+        move(true, r.x, r.y);
+        move(false, r.z, r.w);
     }
     flush();
     // FP64 reductions over the warp, then one atomic per warp
@@ -358,6 +356,7 @@ static awo_status soft_setup(SoftArgs& a, const float* d_h, awo_grid g, const ui
     a.P = p->persistence;
     a.oneP = 1.0f - p->persistence;
     a.R = p->randomness;
+    a.R23 = scaled_randomness(p->randomness);
     a.s = p->step_scale;
     a.D = D;
     a.kD = p->drag_k * D;
