@@ -338,11 +338,12 @@ def run_awo(args, R: Ranks):
     torch.cuda.synchronize()
     st = ov.stats_dict()
     visits = st["total_steps"] + st["n_traj"]
-    # decode and normals (one launch), release (mask, scan, scatter), particle prologue and kernel, then
-    # velocity and mipmap: one launch for both and levels 1..6, one per further level (velocity alone
+    # decode, normals and release mask (one launch), scatter (and a scan of its own above 4096 tiles of 4096
+    # cells), clear, particle prologue and the particle kernel's two instances (one of them ends at once), then
+    # velocity and mipmap: one launch for both and six levels, one per six further levels (velocity alone
     # without a mipmap)
-    lod_launches = 1 if w.lod_levels <= 1 else 1 + max(w.lod_levels - 1 - 6, 0)
-    launches_per_step = 1 + 3 + 3 + lod_launches
+    lod_launches = max(1, -(-(w.lod_levels - 1) // 6))
+    launches_per_step = 1 + 1 + (w.width * w.height > 4096 * 4096) + 4 + lod_launches
 
     peaks_probe = _probe_peaks(torch, awo)
     clocks = ClockSampler(R.local)

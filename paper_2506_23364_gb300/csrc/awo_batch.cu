@@ -47,7 +47,7 @@ struct BatchReq {
 };
 
 struct BatchHeader {
-    SimWorkspace ws[AWO_BATCH_MAX];           // each request's work counter and statistics
+    SimWorkspace ws[AWO_BATCH_MAX];           // each request's work counter (and statistics)
     uint32_t cell_prefix[AWO_BATCH_MAX + 1];  // start records before each request
     uint32_t n_cells[AWO_BATCH_MAX];
     uint32_t check;                           // check_pays of the whole batch
@@ -64,6 +64,8 @@ struct BatchArgs {
     uint32_t n_req;
     uint32_t sim_lanes;  // lanes of one particle launch
     BatchHeader* hdr;
+    unsigned long long* stats;  // 6 per request, stats_step words apart
+    uint32_t stats_step;
     TexelStart* starts;  // one 32-byte slot per release-list entry (CellStarts fill the first half of a request's)
 };
 static_assert(sizeof(BatchArgs) <= 32764, "the request table must fit the kernel parameter block");
@@ -101,7 +103,10 @@ __global__ void __launch_bounds__(AWO_BATCH_MAX) k_batch_prepare(const __grid_co
     // particles for the particle kernel: none for a request with max_steps = 0
     // (every particle capped at its release visit, counted by k_batch_starts)
     s_np[t] = (t < (int)a.n_req && a.r[t].max_steps != 0u) ? (unsigned long long)nc * a.r[t].N : 0ull;
-    if (t < (int)a.n_req) a.hdr->ws[t] = SimWorkspace{};
+    if (t < (int)a.n_req) {
+        a.hdr->ws[t] = SimWorkspace{};
+        for (int i = 0; i < 6; ++i) a.stats[(size_t)t * a.stats_step + i] = 0ull;
+    }
     __syncthreads();
     if (t == 0) {
         unsigned long long total = 0ull, grid = 0ull;
@@ -147,19 +152,13 @@ __global__ void __launch_bounds__(256) k_batch_starts(const __grid_constant__ Ba
         }
         // particles of entries outside the grid are rejected; with max_steps = 0
         // every particle is capped at its release visit (no particle kernel work)
-        unsigned long long* st6 = a.hdr->ws[r].stats;
+        unsigned long long* st6 = a.stats + (size_t)r * a.stats_step;
         if (!ok) atomicAdd(st6 + 5, (unsigned long long)q.N);
         if (ok && q.max_steps == 0u) {
             atomicAdd(st6 + 1, (unsigned long long)q.N);
             atomicAdd(st6 + 3, (unsigned long long)q.N);
         }
     }
-}
-
-// The requests' statistics, gathered for the caller.
-__global__ void __launch_bounds__(256) k_batch_stats(const BatchHeader* hdr, unsigned long long* __restrict__ out, int n)
-{
-    for (int i = threadIdx.x; i < 6 * n; i += blockDim.x) out[i] = hdr->ws[i / 6].stats[i % 6];
 }
 
 static bool tuning_ok(const awo_tuning* t)
@@ -219,6 +218,10 @@ extern "C" awo_status awo_simulate_batched(const awo_sim_request* reqs, int32_t 
     a.sim_lanes = (uint32_t)sm_count() * 1280u;
     a.hdr = static_cast<BatchHeader*>(d_ws);
     a.starts = reinterpret_cast<TexelStart*>(static_cast<char*>(d_ws) + BATCH_HEADER_BYTES);
+    // the kernels count into the caller's statistics where they can
+    const bool direct = d_stats && (((uintptr_t)d_stats) & 7u) == 0;
+    a.stats = direct ? reinterpret_cast<unsigned long long*>(d_stats) : a.hdr->ws[0].stats;
+    a.stats_step = (uint32_t)((direct ? sizeof(awo_sim_stats) : sizeof(SimWorkspace)) / sizeof(unsigned long long));
     SimArgs sim[AWO_BATCH_MAX];  // (no allocation that could throw)
     uint32_t off = 0;
     for (int i = 0; i < n_req; ++i) {
@@ -227,7 +230,8 @@ extern "C" awo_status awo_simulate_batched(const awo_sim_request* reqs, int32_t 
         sim_constants(c, q.d_h, q.grid, &q.params, q.d_count, q.d_maxe, s);
         c.n_cells_dev = a.hdr->n_cells + i;
         c.n_cells_max = q.n_cells_max;
-        c.ws = a.hdr->ws + i;
+        c.next_item = &a.hdr->ws[i].next_item;
+        c.stats = a.stats + (size_t)i * a.stats_step;
         c.starts = a.starts + off;
         c.group = group;
         c.min_idle = refill == AWO_REFILL_WARP ? 32u : 1u;
@@ -264,10 +268,10 @@ extern "C" awo_status awo_simulate_batched(const awo_sim_request* reqs, int32_t 
         after_particles = true;
     }
     if (st != AWO_OK) return st;
-    if (d_stats) {
-        k_batch_stats<<<1, 256, 0, s>>>(a.hdr, reinterpret_cast<unsigned long long*>(d_stats), n_req);
-        return launch_status();
-    }
+    if (d_stats && !direct &&
+        cudaMemcpy2DAsync(d_stats, sizeof(awo_sim_stats), a.hdr->ws[0].stats, sizeof(SimWorkspace), sizeof(awo_sim_stats),
+                          (size_t)n_req, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
+        return AWO_ECUDA;
     return AWO_OK;
 }
 

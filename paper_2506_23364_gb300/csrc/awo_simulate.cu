@@ -68,6 +68,26 @@ __device__ __forceinline__ uint32_t release_count(const SimArgs& a)
     return n;
 }
 
+// Start of a call: the work counter and the statistics zeroed, and n words of
+// both rasters (CLEAR_OUTPUTS; 0 otherwise) -- one launch where three memsets
+// and, for the statistics, a copy at the end of the call took four (2 us each
+// between the kernels of a small call; at 8192^2 as fast as the memsets).
+__global__ void __launch_bounds__(256) k_sim_clear(uint32_t* __restrict__ count, uint32_t* __restrict__ maxe, int64_t n,
+                                                   SimWorkspace* ws, unsigned long long* stats, bool vec4)
+{
+    asm volatile("griddepcontrol.launch_dependents;");
+    const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
+    const int64_t n4 = vec4 ? n / 4 : 0;
+    const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+    for (int64_t q = tid; q < n4; q += stride) {
+        reinterpret_cast<uint4*>(count)[q] = zero;
+        reinterpret_cast<uint4*>(maxe)[q] = zero;
+    }
+    for (int64_t i = 4 * n4 + tid; i < n; i += stride) count[i] = maxe[i] = 0u;
+    if (tid < 6) ws->stats[tid] = stats[tid] = 0ull;
+    if (tid == 6) ws->next_item = 0ull;
+}
+
 // Prologue: per release-list entry, the start record (at its slot in the
 // processing order of awo_particle.cuh) and the release visit of all N particles (count +=
 // N; their energy is 0, so the maximum is unchanged).  Grid-stride over the
@@ -84,6 +104,8 @@ __global__ void __launch_bounds__(256) k_sim_starts(const __grid_constant__ SimA
     const uint32_t nb = n_cells / B;
     __shared__ uint32_t s_sinv;
     if (threadIdx.x == 0) s_sinv = order_stride_inverse(nb);
+    asm volatile("griddepcontrol.launch_dependents;");
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // k_sim_clear
     __syncthreads();
     const uint32_t Sinv = s_sinv;
     // the slot of the thread's entries, advanced per grid stride G (a
@@ -122,10 +144,10 @@ __global__ void __launch_bounds__(256) k_sim_starts(const __grid_constant__ SimA
         bad += __shfl_xor_sync(0xffffffffu, bad, o);
     }
     if ((threadIdx.x & 31) == 0) {
-        if (bad) atomicAdd(&a.ws->stats[5], bad * a.N);
+        if (bad) atomicAdd(&a.stats[5], bad * a.N);
         if (good && a.max_steps == 0u) {
-            atomicAdd(&a.ws->stats[1], good * a.N);
-            atomicAdd(&a.ws->stats[3], good * a.N);
+            atomicAdd(&a.stats[1], good * a.N);
+            atomicAdd(&a.stats[3], good * a.N);
         }
     }
 }
@@ -143,7 +165,7 @@ __global__ void __launch_bounds__(256) k_sim_starts(const __grid_constant__ SimA
 // complete only when all before it are, and what follows on the stream is
 // ordered after every one.  (The same wait at the end of a working block cost
 // 8 registers and 5% on the 8192^2 workload.)
-template <bool TEXELS, bool TEX, bool CHECK>
+template <bool TEXELS, bool TEX, bool PLAIN, bool CHECK>
 __global__ void __launch_bounds__(SIM_THREADS_MAX) k_simulate(const __grid_constant__ SimArgs a)
 {
     extern __shared__ uint32_t s_pool[];  // POOL_WORDS per warp
@@ -162,22 +184,22 @@ __global__ void __launch_bounds__(SIM_THREADS_MAX) k_simulate(const __grid_const
     if (check == CHECK && total > 32ull * blocks * warp) {
         // particles of entries inside the grid (the prologue has counted the others)
         if (blockIdx.x == 0 && threadIdx.x == 0) {
-            const unsigned long long run = total - a.ws->stats[5];
-            a.ws->stats[1] = run;
-            atomicAdd(&a.ws->stats[4], run);
+            const unsigned long long run = total - a.stats[5];
+            a.stats[1] = run;
+            atomicAdd(&a.stats[4], run);
         }
         // particles a warp takes per fetch: a multiple of 32 in [32,
         // SIM_CHUNK_MAX], about total / (warps * SIM_CHUNKS_PER_WARP)
         const unsigned long long even = total / ((unsigned long long)blocks * (blockDim.x >> 5) * SIM_CHUNKS_PER_WARP);
         uint32_t chunk = even > SIM_CHUNK_MAX ? SIM_CHUNK_MAX : max((uint32_t)even & ~31u, 32u);
         if (a.group) chunk = a.group;
-        run_particles<TEXELS, TEX ? 1 : 0, CHECK>(a, total, chunk, a.min_idle, &a.ws->next_item, a.ws->stats,
+        run_particles<TEXELS, TEX ? 1 : 0, CHECK, PLAIN>(a, total, chunk, a.min_idle, a.next_item, a.stats,
                                                   s_pool + warp * POOL_WORDS);
     }
 }
 
-template <bool TEXELS, bool TEX, bool CHECK>
-static awo_status launch_instance(const SimArgs& a, int threads, bool after_particles, cudaStream_t s)
+template <bool TEXELS, bool TEX, bool PLAIN, bool CHECK>
+static awo_status launch_instance(const SimArgs& a, int threads, bool early, cudaStream_t s)
 {
     static int cached[64][3];  // resident blocks per SM, by device and block size (a race writes the same value)
     int dev = 0;
@@ -187,40 +209,33 @@ static awo_status launch_instance(const SimArgs& a, int threads, bool after_part
     int& per_sm = cached[dev][threads == 64 ? 0 : (threads == 128 ? 1 : 2)];
     if (per_sm == 0) {
         int b = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_simulate<TEXELS, TEX, CHECK>, threads, shared) !=
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_simulate<TEXELS, TEX, PLAIN, CHECK>, threads, shared) !=
                 cudaSuccess ||
             b < 1)
             b = 1;
         per_sm = b;
     }
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg;
-    memset(&cfg, 0, sizeof(cfg));
-    cfg.gridDim = dim3((unsigned)(sm_count() * per_sm + 1));
-    cfg.blockDim = dim3((unsigned)threads);
-    cfg.dynamicSmemBytes = shared;
-    cfg.stream = s;
-    cfg.attrs = &attr;
-    cfg.numAttrs = after_particles ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, k_simulate<TEXELS, TEX, CHECK>, a) == cudaSuccess ? launch_status() : AWO_ECUDA;
+    return launch_kernel(k_simulate<TEXELS, TEX, PLAIN, CHECK>, (unsigned)(sm_count() * per_sm + 1), (unsigned)threads, shared,
+                         early, s, a) == cudaSuccess
+               ? launch_status()
+               : AWO_ECUDA;
 }
 
-template <bool TEXELS, bool TEX>
+template <bool TEXELS, bool TEX, bool PLAIN>
 static awo_status launch_both(const SimArgs& a, int threads, bool after_particles, cudaStream_t s)
 {
-    const awo_status st = launch_instance<TEXELS, TEX, true>(a, threads, after_particles, s);
-    return st != AWO_OK ? st : launch_instance<TEXELS, TEX, false>(a, threads, true, s);
+    const awo_status st = launch_instance<TEXELS, TEX, PLAIN, true>(a, threads, after_particles, s);
+    return st != AWO_OK ? st : launch_instance<TEXELS, TEX, PLAIN, false>(a, threads, true, s);
 }
 
 awo_status launch_particles(const SimArgs& a, int threads, bool after_particles, cudaStream_t s)
 {
-    if (a.tg.texels)
-        return a.tex ? launch_both<true, true>(a, threads, after_particles, s)
-                     : launch_both<true, false>(a, threads, after_particles, s);
-    return a.tex ? launch_both<false, true>(a, threads, after_particles, s)
-                 : launch_both<false, false>(a, threads, after_particles, s);
+    const bool plain = a.s == 1.0f && a.kD == 0.0f;
+    auto launch = a.tg.texels ? (a.tex ? (plain ? launch_both<true, true, true> : launch_both<true, true, false>)
+                                       : (plain ? launch_both<true, false, true> : launch_both<true, false, false>))
+                              : (a.tex ? (plain ? launch_both<false, true, true> : launch_both<false, true, false>)
+                                       : (plain ? launch_both<false, false, true> : launch_both<false, false, false>));
+    return launch(a, threads, after_particles, s);
 }
 
 void sim_constants(SimArgs& a, const float* d_h, awo_grid g, const awo_sim_params* p, uint32_t* d_count, float* d_maxe,
@@ -375,52 +390,40 @@ extern "C" awo_status awo_simulate(const float* d_h, awo_grid g, const uint32_t*
     if (ws_bytes < awo_simulate_workspace_bytes(n_cells_max)) return AWO_ENOMEM;
     cudaStream_t s = as_stream(stream);
     SimWorkspace* ws = static_cast<SimWorkspace*>(d_ws);
-    if (cudaMemsetAsync(ws, 0, sizeof(SimWorkspace), s) != cudaSuccess) return AWO_ECUDA;
-    if (p->flags & AWO_SIM_CLEAR_OUTPUTS) {
-        const size_t bytes = (size_t)cells_of(g) * sizeof(uint32_t);
-        if (cudaMemsetAsync(d_count, 0, bytes, s) != cudaSuccess) return AWO_ECUDA;
-        if (cudaMemsetAsync(d_maxe, 0, bytes, s) != cudaSuccess) return AWO_ECUDA;
-    }
+    // the kernels count into the caller's statistics where they can
+    const bool direct = d_stats && (((uintptr_t)d_stats) & 7u) == 0;
 
     SimArgs a;
     sim_constants(a, d_h, g, p, d_count, d_maxe, s);
     a.cells = d_cells;
     a.n_cells_dev = d_n_cells;
     a.n_cells_max = n_cells_max;
-    a.ws = ws;
+    a.next_item = &ws->next_item;
+    a.stats = direct ? reinterpret_cast<unsigned long long*>(d_stats) : ws->stats;
     a.starts = static_cast<char*>(d_ws) + starts_offset();
-    const bool texels = a.tg.texels != 0u;
 
-    if (a.N > 0 && n_cells_max > 0 && a.max_steps == 0u) {  // every particle capped at its release visit
+    const int64_t n_clear = (p->flags & AWO_SIM_CLEAR_OUTPUTS) ? cells_of(g) : 0;
+    const bool vec4 = ((((uintptr_t)d_count) | ((uintptr_t)d_maxe)) & 15u) == 0;
+    k_sim_clear<<<stream_blocks(vec4 ? n_clear / 4 : n_clear, 256), 256, 0, s>>>(
+        d_count, reinterpret_cast<uint32_t*>(d_maxe), n_clear, ws, a.stats, vec4);
+    awo_status st = launch_status();
+    if (st != AWO_OK) return st;
+
+    const bool work = a.N > 0 && n_cells_max > 0;
+    if (work) {
         const unsigned pro_blocks = stream_blocks((int64_t)n_cells_max, 256);
-        if (texels)
-            k_sim_starts<true><<<pro_blocks, 256, 0, s>>>(a);
-        else
-            k_sim_starts<false><<<pro_blocks, 256, 0, s>>>(a);
-        awo_status st = launch_status();
-        if (st != AWO_OK) return st;
-    } else if (a.N > 0 && n_cells_max > 0) {
-        const unsigned pro_blocks = stream_blocks((int64_t)n_cells_max, 256);
-        if (texels)
-            k_sim_starts<true><<<pro_blocks, 256, 0, s>>>(a);
-        else
-            k_sim_starts<false><<<pro_blocks, 256, 0, s>>>(a);
-        if (ev_start && cudaEventRecord(ev_start, s) != cudaSuccess) return AWO_ECUDA;
-        const awo_status launched = launch_particles(a, SIM_THREADS, false, s);
-        if (launched != AWO_OK) return launched;
-        if (ev_stop && cudaEventRecord(ev_stop, s) != cudaSuccess) return AWO_ECUDA;
-    } else if (ev_start) {  // no particle kernel: an empty interval after the call's work
-        if (cudaEventRecord(ev_start, s) != cudaSuccess || cudaEventRecord(ev_stop, s) != cudaSuccess)
-            return AWO_ECUDA;
-    }
-    if (a.N > 0 && n_cells_max > 0 && a.max_steps == 0u && ev_start) {  // prologue only: an empty interval
-        if (cudaEventRecord(ev_start, s) != cudaSuccess || cudaEventRecord(ev_stop, s) != cudaSuccess)
-            return AWO_ECUDA;
-    }
-    if (d_stats) {
-        if (cudaMemcpyAsync(d_stats, ws->stats, sizeof(awo_sim_stats), cudaMemcpyDeviceToDevice, s) !=
+        if (launch_kernel(a.tg.texels ? k_sim_starts<true> : k_sim_starts<false>, pro_blocks, 256, 0, true, s, a) !=
             cudaSuccess)
             return AWO_ECUDA;
     }
+    if (ev_start && cudaEventRecord(ev_start, s) != cudaSuccess) return AWO_ECUDA;
+    if (work && a.max_steps != 0u) {  // else every particle is capped at its release visit
+        st = launch_particles(a, SIM_THREADS, false, s);
+        if (st != AWO_OK) return st;
+    }
+    if (ev_stop && cudaEventRecord(ev_stop, s) != cudaSuccess) return AWO_ECUDA;
+    if (d_stats && !direct && cudaMemcpyAsync(d_stats, ws->stats, sizeof(awo_sim_stats), cudaMemcpyDeviceToDevice, s) !=
+                                  cudaSuccess)
+        return AWO_ECUDA;
     return AWO_OK;
 }
