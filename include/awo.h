@@ -262,7 +262,7 @@ awo_status awo_release_noalloc(const float* d_tan2, awo_grid g, double slope_lo_
  * Workspace: at least awo_simulate_workspace_bytes(n_cells_max) bytes,
  * 16-byte aligned (a work counter, the statistics, and a start record of up
  * to 32 bytes per release-list entry); contents undefined on entry and exit.
- * Gathers: on grids of at least 2^20 cells whose row pitch (4 * width bytes)
+ * Gathers: on grids of at least 2^19 cells whose row pitch (4 * width bytes)
  * and d_h are aligned to the device's texture pitch alignment (32 bytes on
  * GB300), the particle kernel fetches each 2x2 footprint with one texture
  * gather through a texture object that views d_h's 32-bit words (returned
@@ -288,7 +288,7 @@ awo_status awo_simulate(const float* d_h, awo_grid g, const uint32_t* d_cells,
  * (awo_simulate, awo_simulate_batched, the soft-deposit calls) fetch the 2x2
  * footprints of the W x H DEM at d_h by one texture gather through a texture
  * view of the buffer, 0 when they fetch them with four loads (grids under
- * 2^20 cells, a base address or row pitch off the texture alignment, 256
+ * 2^19 cells, a base address or row pitch off the texture alignment, 256
  * views already made, or `stream` being captured).  Like the first launch
  * with that buffer, the call creates the view when one can be made.  Results
  * never depend on the path.  AWO_EINVAL: d_h or texture NULL, or a bad grid.

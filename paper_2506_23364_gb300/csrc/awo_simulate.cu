@@ -31,7 +31,7 @@
 //    lanes of a warp that hit the same cell (__match_any_sync, at the first
 //    move, at both moves of a fresh pair or at every move) was slower wherever
 //    the look is taken (8192^2 18.2 against 17.6 ms, at every move 19.6).
-//  * On grids of at least 2^20 cells the 2x2 footprint of a move is one
+//  * On grids of at least 2^19 cells the 2x2 footprint of a move is one
 //    texture gather through a texture object that views the DEM's words
 //    (clamp addressing is the footprint clamp; indices and weights are still
 //    computed here), in place of four loads, their addresses and clamps.
@@ -294,11 +294,13 @@ void sim_constants(SimArgs& a, const float* d_h, awo_grid g, const awo_sim_param
 // launch stream is being captured into a graph no view is created (an
 // existing one is used, else the loads), so a capture never sees a call it
 // might refuse.  Grids
-// under DEM_VIEW_MIN_CELLS take the loads too: measured on GB300 (particle
-// kernel, texture gathers against loads), 8192^2 -5.5%, 2048^2 -1%, 256^2
-// +4% (a DEM that small stays in L1, where the loads' latency is shorter).
+// under DEM_VIEW_MIN_CELLS take the loads too: measured on GB300 (whole
+// workflow, texture gathers against loads, many / few particles), 768^2 1012
+// against 1085 / 250 against 252 us, 512^2 603 / 604, 165 / 165, 256^2 871 / 892
+// and 380 / 372, 81 / 77 (a DEM that small stays in L1, where the loads' latency
+// is shorter); 8192^2 5.5% less time.
 constexpr int DEM_VIEWS_MAX = 256;
-constexpr int64_t DEM_VIEW_MIN_CELLS = int64_t(1) << 20;
+constexpr int64_t DEM_VIEW_MIN_CELLS = int64_t(1) << 19;
 
 struct DemView {
     const float* h;

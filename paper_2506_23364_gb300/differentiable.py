@@ -86,6 +86,7 @@ class SoftDeposit(torch.autograd.Function):
         (w,) = ctx.saved_tensors
         gt, gw = ctx.prob.backward_raw(ctx.mu, ctx.k, w, gD)
         (sm, dm, vm), (sk, dk, vk) = ctx.meta
-        g_mu = gt[0].to(device=vm, dtype=dm).reshape(sm)
-        g_k = gt[1].to(device=vk, dtype=dk).reshape(sk)
+        gt = gt.to(vm)  # one copy for both where they live together
+        g_mu = gt[0].to(dtype=dm).reshape(sm).clone()
+        g_k = gt[1].to(device=vk, dtype=dk).reshape(sk).clone()
         return g_mu, g_k, gw.to(torch.float32), None
