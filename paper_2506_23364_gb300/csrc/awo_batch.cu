@@ -37,7 +37,7 @@ struct BatchReq {
     const float* h;
     uint32_t* count;
     int W, H;
-    float P, oneP;
+    float P, oneP, s;
     uint32_t max_steps;
     const uint32_t* cells;
     const uint32_t* n_cells_dev;
@@ -62,7 +62,7 @@ static_assert(sizeof(awo_tuning) == 16, "awo_tuning layout (C ABI)");
 struct BatchArgs {
     BatchReq r[AWO_BATCH_MAX];
     uint32_t n_req;
-    uint32_t sim_lanes;  // lanes of one particle launch
+    unsigned long long look_min;  // look_paths of whole-cell steps
     BatchHeader* hdr;
     unsigned long long* stats;  // 6 per request, stats_step words apart
     uint32_t stats_step;
@@ -110,15 +110,17 @@ __global__ void __launch_bounds__(AWO_BATCH_MAX) k_batch_prepare(const __grid_co
     __syncthreads();
     if (t == 0) {
         unsigned long long total = 0ull, grid = 0ull;
+        double paths = 0.0;  // particles over their steps, as in look_paths
         uint32_t cs = 0u;
         for (int r = 0; r < (int)a.n_req; ++r) {
             a.hdr->cell_prefix[r] = cs;
             cs += s_nc[r];
             total += s_np[r];
+            paths += (double)s_np[r] / a.r[r].s;
             grid += a.r[r].n_grid;
         }
         a.hdr->cell_prefix[a.n_req] = cs;
-        a.hdr->check = check_pays(total, a.sim_lanes, grid) ? 1u : 0u;
+        a.hdr->check = paths >= (double)a.look_min || total >= 7ull * grid ? 1u : 0u;  // as check_pays
     }
 }
 
@@ -215,7 +217,7 @@ extern "C" awo_status awo_simulate_batched(const awo_sim_request* reqs, int32_t 
     BatchArgs a;
     memset(&a, 0, sizeof(a));
     a.n_req = (uint32_t)n_req;
-    a.sim_lanes = (uint32_t)sm_count() * 1280u;
+    a.look_min = look_paths(1.0f);
     a.hdr = static_cast<BatchHeader*>(d_ws);
     a.starts = reinterpret_cast<TexelStart*>(static_cast<char*>(d_ws) + BATCH_HEADER_BYTES);
     // the kernels count into the caller's statistics where they can
@@ -243,6 +245,7 @@ extern "C" awo_status awo_simulate_batched(const awo_sim_request* reqs, int32_t 
         b.H = c.H;
         b.P = c.P;
         b.oneP = c.oneP;
+        b.s = c.s;
         b.max_steps = c.max_steps;
         b.cells = q.d_cells;
         b.n_cells_dev = q.d_n_cells;

@@ -176,8 +176,7 @@ __global__ void __launch_bounds__(SIM_THREADS_MAX) k_simulate(const __grid_const
         return;
     }
     const unsigned long long total = (unsigned long long)release_count(a) * a.N;
-    const bool check = a.check ? *a.check != 0u
-                               : check_pays(total, (unsigned long long)blocks * blockDim.x, a.n_grid);
+    const bool check = a.check ? *a.check != 0u : check_pays(total, a.look_min, a.n_grid);
     const uint32_t warp = threadIdx.x >> 5;
     // a few particles: one warp a block, so that they spread over the SMs
     // (parabola, 6144 particles: 149 -> 135 us)
@@ -280,6 +279,7 @@ void sim_constants(SimArgs& a, const float* d_h, awo_grid g, const awo_sim_param
     a.tg.texels = p->release_log2 != 0 ? 1u : 0u;
     a.tex = dem_texture(d_h, g, s);
     a.min_idle = 1u;
+    a.look_min = look_paths(p->step_scale);
 }
 
 // Texture views of DEM buffers for the gathers of k_simulate: a texture

@@ -69,3 +69,16 @@ def test_large_lists_with_and_without_the_look(side, per_lane):
     _, cells = oracle.release(t2, 43.0, 45.0)
     n = -(-per_lane * LANES // cells.size)
     _check(dem, 10.0, cells, dict(traj_per_cell=n, max_steps=60, seed=2))
+
+
+@pytest.mark.parametrize("kw", [{}, dict(step_scale=0.5)])
+@pytest.mark.parametrize("times", [0.85, 0.99, 1.0, 1.01, 1.09, 1.17])
+def test_one_instance_runs_on_either_side_of_the_line(times, kw):
+    """Particle counts around 32 a lane (16 at half steps), few for the grid."""
+    side = 1024
+    y, x = np.mgrid[0:side, 0:side]
+    dem = (9000.0 - 4.0 * x - 3.0 * y).astype(np.float32)
+    total = int(times * 32 * LANES * kw.get("step_scale", 1.0))
+    n = 2048
+    cells = np.arange(3000, 3000 + 17 * (total // n), 17).astype(np.uint32)
+    _check(dem, 10.0, cells, dict(traj_per_cell=n, max_steps=1, seed=8, mu=0.2, **kw))
