@@ -344,7 +344,12 @@ __device__ __forceinline__ uint32_t mask_bits(const uint8_t* __restrict__ mask, 
         const uint4 m = __ldg(reinterpret_cast<const uint4*>(mask + base));
         const uint32_t w[4] = {m.x, m.y, m.z, m.w};
 #pragma unroll
-        for (int k = 0; k < RT_CELLS; ++k) bits |= (((w[k >> 2] >> (8 * (k & 3))) & 0xffu) != 0u ? 1u : 0u) << k;
+        for (int q = 0; q < RT_CELLS / 4; ++q) {
+            // bit 7 of every non-zero byte, then the four bits side by side (bit 8 b + 7 moves to 28 + b; the
+            // product's other terms are distinct bits below 28)
+            const uint32_t set = (w[q] | ((w[q] & 0x7f7f7f7fu) + 0x7f7f7f7fu)) & 0x80808080u;
+            bits |= ((set * 0x00204081u) >> 28) << (4 * q);
+        }
     } else {
 #pragma unroll
         for (int k = 0; k < RT_CELLS; ++k)
@@ -353,14 +358,18 @@ __device__ __forceinline__ uint32_t mask_bits(const uint8_t* __restrict__ mask, 
     return bits;
 }
 
+// The low four bits as 0/1 bytes (bit b to bit 8 b: the product's terms are distinct bits).
+__device__ __forceinline__ uint32_t bytes_of(uint32_t bits)
+{
+    return ((bits & 15u) * 0x00204081u) & 0x01010101u;
+}
+
 // Writes the selection bits as 0/1 bytes (one uint4 when full and aligned).
 __device__ __forceinline__ void store_mask(uint8_t* __restrict__ mask, int64_t base, int64_t n, uint32_t bits)
 {
     uint32_t packed[RT_CELLS / 4];
 #pragma unroll
-    for (int q = 0; q < RT_CELLS / 4; ++q)
-        packed[q] = ((bits >> (4 * q)) & 1u) | (((bits >> (4 * q + 1)) & 1u) << 8) |
-                    (((bits >> (4 * q + 2)) & 1u) << 16) | (((bits >> (4 * q + 3)) & 1u) << 24);
+    for (int q = 0; q < RT_CELLS / 4; ++q) packed[q] = bytes_of(bits >> (4 * q));
     if (base + RT_CELLS <= n && (((uintptr_t)(mask + base)) & 15u) == 0) {
         *reinterpret_cast<uint4*>(mask + base) = make_uint4(packed[0], packed[1], packed[2], packed[3]);
     } else {
@@ -569,6 +578,11 @@ __global__ void __launch_bounds__(RT_THREADS) k_mask_count(const uint8_t* __rest
 // covers SC_RUNS release tiles and starts at the offset of the first: four
 // mask loads in flight per thread and a quarter of the blocks and block scans
 // (measured on GB300, the three release passes at 8192^2: 0.111 -> 0.106 ms).
+// Each thread writes its own indices, a few to a sector.  Collecting a block's
+// in shared memory to write them side by side took 2% longer over the whole
+// terrain of a 4096^2 DEM at 2x, a loop of the warp over its lanes with
+// indices (coalesced too) 6%: nearly every lane has some.  21 us for 67 M
+// texels, 64% of the issue slots, 12 us at the copy rate.
 constexpr int SC_RUNS = 4;
 constexpr int SC_TILE = RT_TILE * SC_RUNS;
 
@@ -589,13 +603,14 @@ __global__ void __launch_bounds__(RT_THREADS) k_mask_scatter(const uint8_t* __re
     int total;
     uint32_t off = (uint32_t)block_exclusive_scan(count, &total) + before;
     if (SUM && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *d_n = before + (uint32_t)total;
+    uint32_t* out = cells + off;
+    const uint32_t b0 = (uint32_t)base;
 #pragma unroll
-    for (int r = 0; r < SC_RUNS; ++r) {
-        uint32_t b = bits[r];
+    for (int half = 0; half < 2; ++half) {
+        uint32_t b = bits[2 * half] | bits[2 * half + 1] << 16;
         while (b) {
-            const int k = __ffs(b) - 1;
-            b &= b - 1;
-            cells[off++] = (uint32_t)(base + r * RT_CELLS + k);
+            *out++ = b0 + 32u * half + (uint32_t)(__ffs(b) - 1);
+            b &= b - 1u;
         }
     }
 }
@@ -759,9 +774,15 @@ __global__ void __launch_bounds__(RT_THREADS) k_release_texture_mask(const float
 // the vertical combination per row (the same operations, in the same order, as
 // k_release_texture_mask).  Group 0 holds the 2^(R-1) rows above the first of
 // those and group H the 2^(R-1) below the last: their centres clamp to the
-// DEM's first and last row.  (Those rows in launches of their own, and a block
-// scan where only its total is wanted: 61 us for the mask of a 4096^2 DEM at
-// 2x.)
+// DEM's first and last row.  The runs at a row's ends are not texel by texel
+// but differ only in the weights of their 2^(R-1) clamped texels and in the
+// columns of their outer loads (one slow lane in every block had the other
+// warps wait at its barrier, 7.6 warps an issue), and the texels are selected
+// as bytes of the mask's words: 46 -> 36 us for the mask of a 4096^2 DEM at
+// 2x, 89 -> 71 us for the whole terrain of a 2048^2 one at 4x.  Issue slots
+// bound it (16 warp instructions per 32 texels before; HBM would take 20 us).
+// (The edge rows in launches of their own and a block scan where only its
+// total is wanted: 61 us.)
 template <int R, bool VEC>
 __global__ void __launch_bounds__(RT_THREADS) k_release_texture_rows(const float* __restrict__ tan2, int W, int H,
                                                                      uint32_t Wr, int64_t n, float scale,
@@ -778,7 +799,7 @@ __global__ void __launch_bounds__(RT_THREADS) k_release_texture_rows(const float
     const int dj = j + 1 < H ? W : 0;          // to the row below, clamped
     const uint32_t b0 = group == 0 ? 0u : (uint32_t)j * ROWS + HALF;  // first texture row of the group
     const uint32_t a = blockIdx.x * (uint32_t)RT_TILE + threadIdx.x * (uint32_t)RT_CELLS;
-    const float hm1 = __int2float_rn(H - 1), wm1 = __int2float_rn(W - 1);
+    const float hm1 = __int2float_rn(H - 1);
     float oy[ROWS], fy[ROWS];
 #pragma unroll
     for (int r = 0; r < ROWS; ++r) {
@@ -787,66 +808,68 @@ __global__ void __launch_bounds__(RT_THREADS) k_release_texture_rows(const float
         oy[r] = __fsub_rn(1.0f, fy[r]);
     }
     const int row = j * W;
-    uint32_t bits[ROWS];
+    uint32_t sel[ROWS][RT_CELLS / 4];  // the run's mask bytes
 #pragma unroll
-    for (int r = 0; r < ROWS; ++r) bits[r] = 0u;
+    for (int r = 0; r < ROWS; ++r)
+#pragma unroll
+        for (int q = 0; q < RT_CELLS / 4; ++q) sel[r][q] = 0u;
     const int A = (int)(a >> R);
-    if (A + T::DMIN >= 0 && A + T::DMAX + 1 <= W - 2) {
-        float top[T::NC], bot[T::NC];
-        const float* p = tan2 + row + A;
+    const bool first = A == 0, last = A + T::DMAX + 1 == W;  // the runs at the row's ends
+    float top[T::NC], bot[T::NC];
+    const float* p = tan2 + row + A;
 #pragma unroll
-        for (int i = T::DMIN; i <= T::DMAX + 1; ++i) {
-            const int g = i & ~3;
-            const bool whole = VEC && g >= T::DMIN && g + 3 <= T::DMAX + 1;
-            if (whole && i == g) {
-                const float4 qt = __ldg(reinterpret_cast<const float4*>(p + i));
-                const float4 qb = __ldg(reinterpret_cast<const float4*>(p + dj + i));
-                top[i - T::DMIN] = qt.x, top[i - T::DMIN + 1] = qt.y, top[i - T::DMIN + 2] = qt.z,
-                              top[i - T::DMIN + 3] = qt.w;
-                bot[i - T::DMIN] = qb.x, bot[i - T::DMIN + 1] = qb.y, bot[i - T::DMIN + 2] = qb.z,
-                              bot[i - T::DMIN + 3] = qb.w;
-            } else if (!whole) {
-                top[i - T::DMIN] = __ldg(p + i);
-                bot[i - T::DMIN] = __ldg(p + dj + i);
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < RT_CELLS; ++k) {
-            const int c = T::delta(k) - T::DMIN;
-            const float fx = T::frac(k), ox = T::one_minus_frac(k);
-            const float tp = __fadd_rn(__fmul_rn(top[c], ox), __fmul_rn(top[c + 1], fx));
-            const float bt = __fadd_rn(__fmul_rn(bot[c], ox), __fmul_rn(bot[c + 1], fx));
-#pragma unroll
-            for (int r = 0; r < ROWS; ++r) {
-                const float Tk = __fadd_rn(__fmul_rn(tp, oy[r]), __fmul_rn(bt, fy[r]));
-                bits[r] |= ((t_lo <= Tk && Tk <= t_hi) ? 1u : 0u) << k;
-            }
-        }
-    } else {
-        // the run touches a row end: texel by texel, columns clamped as in the general path
-#pragma unroll 1
-        for (int k = 0; k < RT_CELLS; ++k) {
-            const float u = texel_centre(a + (uint32_t)k, scale, wm1);
-            const int i0 = __float2int_rd(u);
-            const float fx = __fsub_rn(u, __int2float_rn(i0));
-            const int o = row + i0, di = i0 + 1 < W ? 1 : 0;
-            const float t00 = __ldg(tan2 + o), t10 = __ldg(tan2 + o + di);
-            const float t01 = __ldg(tan2 + o + dj), t11 = __ldg(tan2 + o + dj + di);
-            const float ox = __fsub_rn(1.0f, fx);
-            const float tp = __fadd_rn(__fmul_rn(t00, ox), __fmul_rn(t10, fx));
-            const float bt = __fadd_rn(__fmul_rn(t01, ox), __fmul_rn(t11, fx));
-#pragma unroll
-            for (int r = 0; r < ROWS; ++r) {
-                const float Tk = __fadd_rn(__fmul_rn(tp, oy[r]), __fmul_rn(bt, fy[r]));
-                bits[r] |= ((t_lo <= Tk && Tk <= t_hi) ? 1u : 0u) << k;
-            }
+    for (int i = T::DMIN; i <= T::DMAX + 1; ++i) {
+        const int g = i & ~3;
+        const bool whole = VEC && g >= 0 && g + 3 <= T::DMAX;
+        if (whole && i == g) {
+            const float4 qt = __ldg(reinterpret_cast<const float4*>(p + i));
+            const float4 qb = __ldg(reinterpret_cast<const float4*>(p + dj + i));
+            top[i - T::DMIN] = qt.x, top[i - T::DMIN + 1] = qt.y, top[i - T::DMIN + 2] = qt.z,
+                          top[i - T::DMIN + 3] = qt.w;
+            bot[i - T::DMIN] = qb.x, bot[i - T::DMIN + 1] = qb.y, bot[i - T::DMIN + 2] = qb.z,
+                          bot[i - T::DMIN + 3] = qb.w;
+        } else if (!whole) {
+            const int c = min(max(i, -A), W - 1 - A);  // inside the row
+            top[i - T::DMIN] = __ldg(p + c);
+            bot[i - T::DMIN] = __ldg(p + dj + c);
         }
     }
+#pragma unroll
+    for (int k = 0; k < RT_CELLS; ++k) {
+        const int c = T::delta(k) - T::DMIN;
+        float fx = T::frac(k), ox = T::one_minus_frac(k);
+        float tl = top[c], tr = top[c + 1], bl = bot[c], br = bot[c + 1];
+        if (k < HALF && first) {  // centre clamped to column 0: weights 1 and 0 of columns 0 and 1
+            fx = 0.0f, ox = 1.0f;
+            tl = top[c + 1], tr = top[c + 2], bl = bot[c + 1], br = bot[c + 2];
+        }
+        if (k >= RT_CELLS - HALF && last) {  // clamped to column W - 1: weights 1 and 0 of that column
+            fx = 0.0f, ox = 1.0f;
+            tr = tl, br = bl;
+        }
+        const float tp = __fadd_rn(__fmul_rn(tl, ox), __fmul_rn(tr, fx));
+        const float bt = __fadd_rn(__fmul_rn(bl, ox), __fmul_rn(br, fx));
+#pragma unroll
+        for (int r = 0; r < ROWS; ++r) {
+            const float Tk = __fadd_rn(__fmul_rn(tp, oy[r]), __fmul_rn(bt, fy[r]));
+            if (t_lo <= Tk && Tk <= t_hi) sel[r][k / 4] |= 1u << (8 * (k % 4));
+        }
+    }
+    const bool aligned = ((uintptr_t)mask & 15u) == 0;  // and so every run: rows are whole tiles
     __shared__ int s_count[ROWS][RT_THREADS / 32];
 #pragma unroll
     for (int r = 0; r < ROWS; ++r) {
-        if (!edge || r < HALF) store_mask(mask, (int64_t)(b0 + r) * Wr + a, n, bits[r]);
-        const int c = __reduce_add_sync(0xffffffffu, __popc(bits[r]));
+        if (!edge || r < HALF) {
+            uint8_t* m = mask + (size_t)(b0 + r) * Wr + a;
+            if (aligned) {
+                *reinterpret_cast<uint4*>(m) = make_uint4(sel[r][0], sel[r][1], sel[r][2], sel[r][3]);
+            } else {
+#pragma unroll
+                for (int k = 0; k < RT_CELLS; ++k) m[k] = (uint8_t)(sel[r][k / 4] >> (8 * (k % 4)));
+            }
+        }
+        const uint32_t bytes = sel[r][0] + sel[r][1] + sel[r][2] + sel[r][3];  // at most 4 each
+        const int c = __reduce_add_sync(0xffffffffu, (int)((bytes * 0x01010101u) >> 24));
         if ((threadIdx.x & 31) == 0) s_count[r][threadIdx.x >> 5] = c;
     }
     __syncthreads();

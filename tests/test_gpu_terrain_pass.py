@@ -70,3 +70,41 @@ def test_texture_row_groups_on_few_rows(r, W, H):
     mask, texels = oracle.release_texture(t2, r, 20.0, 60.0)
     assert np.array_equal(ov.mask.cpu().numpy().ravel(), np.asarray(mask).ravel())
     assert np.array_equal(ov.release_cells(), texels)
+
+
+@pytest.mark.parametrize("tan2_off,mask_off", [(0, 0), (1, 0), (0, 3)])
+@pytest.mark.parametrize("r,W,H", [(1, 2048, 4), (1, 4096, 2), (2, 1024, 5), (2, 3072, 2)])
+def test_texture_row_groups_ends_and_offsets(r, W, H, tan2_off, mask_off):
+    """Runs at the row ends, the vector and scalar loads and stores, values that no weight may touch."""
+    rng = np.random.default_rng(W + H)
+    t2 = (rng.random((H, W)) * 2.0).astype(np.float32)
+    vals = np.array([0.0, 1e-42, 3e38, np.inf, np.nan, 1.0], np.float32)
+    for col in (0, 1, 2, W - 3, W - 2, W - 1, 7, 8, W // 2):
+        t2[:, col] = vals[rng.integers(0, vals.size, H)]
+    buf = torch.zeros(W * H + tan2_off, device="cuda")
+    d_t2 = buf[tan2_off:]
+    d_t2.copy_(torch.from_numpy(t2.ravel()))
+    g = awo.grid(W, H, 10.0)
+    wr, hr = awo.awo_release_texture_dims(g, r)
+    mask = torch.full((wr * hr + mask_off,), 9, dtype=torch.uint8, device="cuda")
+    texels = torch.zeros(wr * hr, dtype=torch.int32, device="cuda")
+    n = torch.zeros(1, dtype=torch.int32, device="cuda")
+    ws = torch.empty(awo.awo_release_texture_workspace_bytes(g, r), dtype=torch.uint8, device="cuda")
+    awo.awo_release_texture(d_t2, g, r, 30.0, 50.0, mask[mask_off:], texels, n, ws)
+    torch.cuda.synchronize()
+    want_mask, want = oracle.release_texture(t2, r, 30.0, 50.0)
+    assert np.array_equal(mask[mask_off:].cpu().numpy(), np.asarray(want_mask).ravel())
+    assert np.array_equal(texels[:int(n)].cpu().numpy().view(np.uint32), want)
+
+
+@pytest.mark.parametrize("size", [16, 4096, 16384, 16387, 40000])
+def test_mask_bytes_of_any_value(size):
+    rng = np.random.default_rng(size)
+    m = np.where(rng.random(size) < 0.5, 0, rng.choice([1, 2, 0x7f, 0x80, 0xff], size)).astype(np.uint8)
+    g = awo.grid(size, 1, 10.0)
+    cells = torch.zeros(size, dtype=torch.int32, device="cuda")
+    n = torch.zeros(1, dtype=torch.int32, device="cuda")
+    ws = torch.empty(awo.awo_release_workspace_bytes(g), dtype=torch.uint8, device="cuda")
+    awo.awo_release_from_mask(torch.from_numpy(m).cuda(), g, cells, n, ws)
+    torch.cuda.synchronize()
+    assert np.array_equal(cells[:int(n)].cpu().numpy(), np.flatnonzero(m))
