@@ -60,15 +60,16 @@ ALG_OPS_PER_VISIT = 126
 #   lts_frac: lts__throughput.avg.pct_of_peak_sustained_elapsed / 100, the L2's
 #     own utilisation against its peak -- the L2 gather/reduction roofline
 #     fraction of the kernel
-#   red_sectors, read_sectors: lts__t_sectors_srcunit_tex_op_red.sum and
-#     lts__t_sectors_srcunit_tex_op_read.sum (the visits' reductions, and the
-#     footprint reads that miss in the L1/texture cache, as the SMs send them)
+#   red_sectors, read_sectors: l1tex__t_sectors_pipe_lsu_mem_global_op_red.sum,
+#     and the texture and load sectors less their lookup hits (the visits'
+#     reductions, and the footprints and maxima that miss in the L1/texture
+#     cache, as the SMs send them)
 #   atomic_busy: lts__d_atomic_input_cycles_active.avg.pct_of_peak_sustained_elapsed
 #     / 100, the share of cycles the L2's reduction units take input
 KERNEL_COUNTERS: dict[str, dict[str, float]] = {
-    "21bee4ee6bfef80c": {"dram": (917.063680e6 + 189.185280e6) / 1754008332, "lts_frac": 0.77099731,
-                         "red_sectors": 2177706165 / 1754008332, "read_sectors": 32575163 / 1754008332,
-                         "atomic_busy": 0.52413501},
+    "98baa25ce7c2d225": {"dram": (1138.118912e6 + 177.382144e6) / 1754008332, "lts_frac": 0.5105,
+                         "red_sectors": 1191971881 / 1754008332, "read_sectors": 38551609 / 1754008332,
+                         "atomic_busy": 0.3353},
 }
 
 
