@@ -73,8 +73,8 @@ __global__ void k_decode_u16(const uint16_t* __restrict__ q, int64_t n, float sc
 // run).  When rows are 16-byte aligned (W % 4 == 0 and aligned buffers) the
 // run's heights, the rows above and below and the outputs move as float4;
 // the two horizontal neighbours outside the run are scalar loads (L1 hits)
-// (k_normals_tiles).  Otherwise each cell is handled alone with the same
-// arithmetic (k_normals).
+// (k_normals_tiles).  Otherwise each thread takes single cells, side by side
+// in a warp, with the same arithmetic (k_normals_cells).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void normal_of(float gx, float gy, float& nx, float& ny, float& nz, float& t2)
 {
@@ -213,46 +213,6 @@ __device__ __forceinline__ float4 normals_run(const NormalsArgs<FROM_U16>& a, co
     return t;
 }
 
-// The cells one by one: ragged rows and unaligned buffers.
-template <bool FROM_U16>
-__global__ void __launch_bounds__(256) k_normals(const __grid_constant__ NormalsArgs<FROM_U16> a)
-{
-    const int W = a.W, H = a.H;
-    const int64_t plane = (int64_t)W * H;
-    const uint32_t runs = (uint32_t)((W + 3) >> 2);
-    const uint32_t items = runs * (uint32_t)H;
-    const SpanDiv d = span_div(a.cs);
-    for (uint32_t it = blockIdx.x * blockDim.x + threadIdx.x; it < items; it += gridDim.x * blockDim.x) {
-        const int y = (int)(it / runs);
-        const int x0 = (int)(it - (uint32_t)y * runs) * 4;
-        const int yl = y > 0 ? y - 1 : 0, yr = y < H - 1 ? y + 1 : H - 1;
-        const float deny = yr - yl == 2 ? d.den2 : d.den1, rdeny = yr - yl == 2 ? d.rden2 : d.rden1;
-        const int64_t row = (int64_t)y * W;
-        const int x_end = x0 + 4 < W ? x0 + 4 : W;
-        for (int x = x0; x < x_end; ++x) {
-            const int xl = x > 0 ? x - 1 : 0, xr = x < W - 1 ? x + 1 : W - 1;
-            float gx = 0.0f, gy = 0.0f;
-            if (xr > xl)
-                gx = div_rn_by_rcp<true>(__fsub_rn(a.h.at(row + xr), a.h.at(row + xl)), xr - xl == 2 ? d.den2 : d.den1,
-                                         xr - xl == 2 ? d.rden2 : d.rden1);
-            if (yr > yl)
-                gy = div_rn_by_rcp<true>(__fsub_rn(a.h.at((int64_t)yr * W + x), a.h.at((int64_t)yl * W + x)), deny,
-                                         rdeny);
-            float nx, ny, nz, t2;
-            normal_of(gx, gy, nx, ny, nz, t2);
-            const int64_t i = row + x;
-            if (FROM_U16) a.h_out[i] = a.h.at(i);
-            if (a.nrm) {
-                a.nrm[i] = nx;
-                a.nrm[plane + i] = ny;
-                a.nrm[2 * plane + i] = nz;
-            }
-            if (a.tan2) a.tan2[i] = t2;
-            if (a.slope_deg) a.slope_deg[i] = slope_deg_of(t2);
-        }
-    }
-}
-
 // ---------------------------------------------------------------------------
 // b. release selection, deterministic and ordered.
 //   1. mask + per-tile count   (tile = RT_THREADS * RT_CELLS cells)
@@ -292,17 +252,18 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int* total)
     return base + incl - v;
 }
 
-// Sum of v over the block, in thread 0 (call once per kernel: one barrier).
+// Sum of v over the block of THREADS, in thread 0 (call once per kernel: one barrier).
+template <int THREADS = RT_THREADS>
 __device__ __forceinline__ uint32_t block_total(int v)
 {
-    __shared__ int warp_total[RT_THREADS / 32];
+    __shared__ int warp_total[THREADS / 32];
     const int t = __reduce_add_sync(0xffffffffu, v);
     if ((threadIdx.x & 31) == 0) warp_total[threadIdx.x >> 5] = t;
     __syncthreads();
     int total = 0;
     if (threadIdx.x == 0) {
 #pragma unroll
-        for (int w = 0; w < RT_THREADS / 32; ++w) total += warp_total[w];
+        for (int w = 0; w < THREADS / 32; ++w) total += warp_total[w];
     }
     return (uint32_t)total;
 }
@@ -451,6 +412,76 @@ __global__ void __launch_bounds__(RT_THREADS) k_normals_tiles(const __grid_const
     }
     if (tile_count) {
         const uint32_t total = block_total(count);
+        if (threadIdx.x == 0) tile_count[blockIdx.x] = total;
+    }
+}
+
+// The same for any width and alignment: single cells, a warp's side by side,
+// so that every load and store is coalesced whatever the rows' alignment
+// (four consecutive cells a thread, one after the other, touched each sector
+// four times and took 3325 x 4197 with the release pass 238 -> 94 us, 7.7
+// times the aligned kernel's time a cell before and 1.8 now: 3.3 TB/s, bound
+// by issue and by the five loads of a cell).  512 threads: 256 or 1024 took
+// 626 x 422 19.1 -> 20-22 us.  A block takes `span` cells: a release tile when
+// it counts one.
+constexpr int NC_THREADS = 512;
+
+template <bool FROM_U16>
+__global__ void __launch_bounds__(NC_THREADS) k_normals_cells(const __grid_constant__ NormalsArgs<FROM_U16> a,
+                                                                uint32_t span, float t_lo, float t_hi,
+                                                                uint8_t* __restrict__ mask,
+                                                                uint32_t* __restrict__ tile_count)
+{
+    const uint32_t W = (uint32_t)a.W, H = (uint32_t)a.H, n = W * H;  // below 2^31
+    const SpanDiv d = span_div(a.cs);
+    const bool spans = d.den1 >= 0x1p-60f && d.den2 <= 0x1p60f;
+    const uint32_t first = blockIdx.x * span;
+    const uint32_t y_first = first / W, x_first = first - y_first * W;
+    int count = 0;
+#pragma unroll 2
+    for (uint32_t k = threadIdx.x; k < span; k += NC_THREADS) {
+        const uint32_t i = first + k;
+        if (i >= n) break;
+        uint32_t y = y_first, x = x_first + k;
+        if (x >= W) {
+            const uint32_t rows = x / W;
+            y += rows;
+            x -= rows * W;
+        }
+        const uint32_t xl = x > 0u ? i - 1u : i, xr = x + 1u < W ? i + 1u : i;
+        const uint32_t yl = y > 0u ? i - W : i, yr = y + 1u < H ? i + W : i;
+        const float dx = __fsub_rn(a.h.at(xr), a.h.at(xl)), dy = __fsub_rn(a.h.at(yr), a.h.at(yl));
+        if (FROM_U16) a.h_out[i] = a.h.at(i);
+        const bool two_x = xr - xl == 2u, two_y = yr - yl == 2u * W;
+        const float denx = two_x ? d.den2 : d.den1, rdx = two_x ? d.rden2 : d.rden1;
+        const float deny = two_y ? d.den2 : d.den1, rdy = two_y ? d.rden2 : d.rden1;
+        // one range test for both divisions and the root, as in normals_run
+        const uint32_t bx = __float_as_uint(dx) & 0x7fffffffu, by = __float_as_uint(dy) & 0x7fffffffu;
+        const float gx = with_sign(div_rn_mid(dx, denx, rdx), dx), gy = with_sign(div_rn_mid(dy, deny, rdy), dy);
+        float t2 = __fadd_rn(__fmul_rn(gx, gx), __fmul_rn(gy, gy));
+        const float top = __fadd_rn(t2, 1.0f);
+        float nz = rcp_sqrt_mid(top);
+        float nx = __fmul_rn(-gx, nz), ny = __fmul_rn(-gy, nz);
+        if (!(min(bx - 1u, by - 1u) >= DIV_LOW - 1u && max(bx, by) <= DIV_HIGH && top <= 0x1p100f && spans)) {
+            const float ex = xr > xl ? div_rn_by_rcp<true>(dx, denx, rdx) : 0.0f;
+            const float ey = yr > yl ? div_rn_by_rcp<true>(dy, deny, rdy) : 0.0f;
+            normal_of(ex, ey, nx, ny, nz, t2);
+        }
+        if (a.nrm) {
+            a.nrm[i] = nx;
+            a.nrm[(size_t)n + i] = ny;
+            a.nrm[2 * (size_t)n + i] = nz;
+        }
+        if (a.tan2) a.tan2[i] = t2;
+        if (a.slope_deg) a.slope_deg[i] = slope_deg_of(t2);
+        if (tile_count) {
+            const uint32_t sel = t_lo <= t2 && t2 <= t_hi ? 1u : 0u;
+            if (mask) mask[i] = (uint8_t)sel;
+            count += (int)sel;
+        }
+    }
+    if (tile_count) {
+        const uint32_t total = block_total<NC_THREADS>(count);
         if (threadIdx.x == 0) tile_count[blockIdx.x] = total;
     }
 }
@@ -687,8 +718,8 @@ __device__ __forceinline__ uint32_t texel_run_bits(const float* __restrict__ tan
     return bits;
 }
 
-// R >= 0: runs in one row away from the row ends take texel_run_bits; the
-// rest (and every run when R < 0, written R = -1) the general per-texel path.
+// Runs in one row away from the row ends take texel_run_bits; the rest the
+// general per-texel path.
 // VEC as in texel_run_bits (host-checked alignment of tan2 and W; R <= 2).
 template <int R, bool VEC>
 __global__ void __launch_bounds__(RT_THREADS) k_release_texture_mask(const float* __restrict__ tan2, int W, int H,
@@ -714,10 +745,10 @@ __global__ void __launch_bounds__(RT_THREADS) k_release_texture_mask(const float
     int row = j0 * W, dj = j0 + 1 < H ? W : 0;
     uint32_t bits = 0u;
     bool done = false;
-    if (R >= 0 && base + RT_CELLS <= n32 && a + RT_CELLS <= Wr) {
-        const int A = (int)(a >> (R >= 0 ? R : 0));
-        if (A + TexRun<(R >= 0 ? R : 0)>::DMIN >= 0 && A + TexRun<(R >= 0 ? R : 0)>::DMAX + 1 <= W - 2) {
-            bits = texel_run_bits<(R >= 0 ? R : 0), VEC>(tan2, row, dj, A, oy, fy, t_lo, t_hi);
+    if (base + RT_CELLS <= n32 && a + RT_CELLS <= Wr) {
+        const int A = (int)(a >> R);
+        if (A + TexRun<R>::DMIN >= 0 && A + TexRun<R>::DMAX + 1 <= W - 2) {
+            bits = texel_run_bits<R, VEC>(tan2, row, dj, A, oy, fy, t_lo, t_hi);
             done = true;
         }
     }
@@ -762,6 +793,49 @@ __global__ void __launch_bounds__(RT_THREADS) k_release_texture_mask(const float
     store_mask(mask, base, n, bits);
     const uint32_t total = block_total(__popc(bits));
     if (threadIdx.x == 0) tile_count[tile] = total;
+}
+
+// Coarser textures (R < 0), any width: single texels, a warp's side by side,
+// with the footprint of its centre.  (A run of 16 texels a thread, whose
+// footprints share nothing here, was a chain of 16 loads: terrain of 2112 x
+// 1344 at 1/2 40.3 -> 27.5 us, of 3001 x 2999 at 1/4, normals included, 158 ->
+// 69 us.  On finer textures the runs' shared loads win: 3325 x 4197 at 2x 189
+// against 263 us.)
+__global__ void __launch_bounds__(NC_THREADS) k_release_texture_texels(const float* __restrict__ tan2, int W, int H,
+                                                                         uint32_t Wr, uint32_t n, float scale,
+                                                                         float t_lo, float t_hi,
+                                                                         uint8_t* __restrict__ mask,
+                                                                         uint32_t* __restrict__ tile_count)
+{
+    const float wm1 = __int2float_rn(W - 1), hm1 = __int2float_rn(H - 1);
+    const uint32_t first = blockIdx.x * (uint32_t)RT_TILE;
+    const uint32_t b_first = first / Wr, a_first = first - b_first * Wr;
+    int count = 0;
+#pragma unroll 4
+    for (uint32_t k = threadIdx.x; k < (uint32_t)RT_TILE; k += NC_THREADS) {
+        if (first + k >= n) break;
+        uint32_t b = b_first, a = a_first + k;
+        if (a >= Wr) {
+            const uint32_t rows = a / Wr;
+            b += rows;
+            a -= rows * Wr;
+        }
+        const float u = texel_centre(a, scale, wm1), v = texel_centre(b, scale, hm1);
+        const int i0 = __float2int_rd(u), j0 = __float2int_rd(v);
+        const float fx = __fsub_rn(u, __int2float_rn(i0)), fy = __fsub_rn(v, __int2float_rn(j0));
+        const float ox = __fsub_rn(1.0f, fx), oy = __fsub_rn(1.0f, fy);
+        const int o = j0 * W + i0, di = i0 + 1 < W ? 1 : 0, dj = j0 + 1 < H ? W : 0;
+        const float t00 = __ldg(tan2 + o), t10 = __ldg(tan2 + o + di);
+        const float t01 = __ldg(tan2 + o + dj), t11 = __ldg(tan2 + o + dj + di);
+        const float top = __fadd_rn(__fmul_rn(t00, ox), __fmul_rn(t10, fx));
+        const float bot = __fadd_rn(__fmul_rn(t01, ox), __fmul_rn(t11, fx));
+        const float T = __fadd_rn(__fmul_rn(top, oy), __fmul_rn(bot, fy));
+        const uint32_t sel = t_lo <= T && T <= t_hi ? 1u : 0u;
+        mask[first + k] = (uint8_t)sel;
+        count += (int)sel;
+    }
+    const uint32_t total = block_total<NC_THREADS>(count);
+    if (threadIdx.x == 0) tile_count[blockIdx.x] = total;
 }
 
 // Rows that share their tan^2 rows (R = 1, 2): texture rows b = 2^R j + 2^(R-1)
@@ -932,8 +1006,13 @@ static awo_status launch_normals(const NormalsArgs<FROM_U16>& a, awo_grid g, boo
     if (aligned)
         k_normals_tiles<FROM_U16><<<(unsigned)((n + RT_TILE - 1) / RT_TILE), RT_THREADS, 0, s>>>(a, 0.0f, 0.0f, nullptr,
                                                                                                  nullptr);
-    else
-        k_normals<FROM_U16><<<stream_blocks((int64_t)((g.width + 3) / 4) * g.height, 256), 256, 0, s>>>(a);
+    else {
+        // a quarter of a tile a block while whole tiles would leave SMs with few blocks (501 x 151: parabola
+        // workflow 125.7 -> 122.2 us; 3001 x 2999 the other way round 75.2 -> 69.2 us)
+        const int64_t span = n >= (int64_t)sm_count() * 4 * RT_TILE ? RT_TILE : RT_TILE / 4;
+        k_normals_cells<FROM_U16><<<(unsigned)((n + span - 1) / span), NC_THREADS, 0, s>>>(a, (uint32_t)span, 0.0f,
+                                                                                          0.0f, nullptr, nullptr);
+    }
     return launch_status();
 }
 
@@ -1010,17 +1089,19 @@ extern "C" awo_status awo_release(const float* d_tan2, awo_grid g, double slope_
     return launch_status();
 }
 
-// a0 + a1 + b: the fused pass where rows are 16-byte aligned, else the calls
-// one after the other.
+// a0 + a1 + b, with the release mask and counts taken in the normals' pass.
 template <bool FROM_U16>
-static awo_status normals_release(const NormalsArgs<FROM_U16>& a, awo_grid g, double lo, double hi, uint8_t* d_mask,
-                                  uint32_t* d_cells, uint32_t* d_n, void* d_ws, cudaStream_t s)
+static awo_status normals_release(const NormalsArgs<FROM_U16>& a, awo_grid g, bool aligned, double lo, double hi,
+                                  uint8_t* d_mask, uint32_t* d_cells, uint32_t* d_n, void* d_ws, cudaStream_t s)
 {
     const int64_t n = cells_of(g);
     const int tiles = (int)((n + RT_TILE - 1) / RT_TILE);
     uint32_t* tile_count = static_cast<uint32_t*>(d_ws);
     const float t_lo = tan2_of_degrees(lo), t_hi = tan2_of_degrees(hi);
-    k_normals_tiles<FROM_U16><<<tiles, RT_THREADS, 0, s>>>(a, t_lo, t_hi, d_mask, tile_count);
+    if (aligned)
+        k_normals_tiles<FROM_U16><<<tiles, RT_THREADS, 0, s>>>(a, t_lo, t_hi, d_mask, tile_count);
+    else
+        k_normals_cells<FROM_U16><<<tiles, NC_THREADS, 0, s>>>(a, (uint32_t)RT_TILE, t_lo, t_hi, d_mask, tile_count);
     scan_and_scatter(a.tan2, d_mask, n, tiles, t_lo, t_hi, tile_count, tile_count + tiles, d_cells, d_n, s);
     return launch_status();
 }
@@ -1031,15 +1112,12 @@ extern "C" awo_status awo_normals_release(const float* d_h, awo_grid g, float* d
                                           size_t ws_bytes, void* stream)
 {
     if (!d_h) return AWO_EINVAL;
-    awo_status st = release_args(d_tan2, g, slope_lo_deg, slope_hi_deg, d_cells, d_n, d_ws, ws_bytes);
+    const awo_status st = release_args(d_tan2, g, slope_lo_deg, slope_hi_deg, d_cells, d_n, d_ws, ws_bytes);
     if (st != AWO_OK) return st;
-    if (runs_aligned(g, d_h, 16, d_normal, d_tan2, d_slope_deg, nullptr, d_mask))
-        return normals_release(
-            NormalsArgs<false>{{d_h, 1.0f}, g.width, g.height, g.cell_size, d_normal, d_tan2, d_slope_deg, nullptr}, g,
-            slope_lo_deg, slope_hi_deg, d_mask, d_cells, d_n, d_ws, as_stream(stream));
-    st = awo_normals(d_h, g, d_normal, d_tan2, d_slope_deg, stream);
-    return st != AWO_OK ? st
-                        : awo_release(d_tan2, g, slope_lo_deg, slope_hi_deg, d_mask, d_cells, d_n, d_ws, ws_bytes, stream);
+    return normals_release(
+        NormalsArgs<false>{{d_h, 1.0f}, g.width, g.height, g.cell_size, d_normal, d_tan2, d_slope_deg, nullptr}, g,
+        runs_aligned(g, d_h, 16, d_normal, d_tan2, d_slope_deg, nullptr, d_mask), slope_lo_deg, slope_hi_deg, d_mask,
+        d_cells, d_n, d_ws, as_stream(stream));
 }
 
 extern "C" awo_status awo_normals_u16_release(const uint16_t* d_q, awo_grid g, float scale, float* d_h, float* d_normal,
@@ -1048,15 +1126,12 @@ extern "C" awo_status awo_normals_u16_release(const uint16_t* d_q, awo_grid g, f
                                               void* d_ws, size_t ws_bytes, void* stream)
 {
     if (!d_q || !d_h || !(scale > 0.0f) || !(scale < 3.0e38f)) return AWO_EINVAL;
-    awo_status st = release_args(d_tan2, g, slope_lo_deg, slope_hi_deg, d_cells, d_n, d_ws, ws_bytes);
+    const awo_status st = release_args(d_tan2, g, slope_lo_deg, slope_hi_deg, d_cells, d_n, d_ws, ws_bytes);
     if (st != AWO_OK) return st;
-    if (runs_aligned(g, d_q, 8, d_normal, d_tan2, d_slope_deg, d_h, d_mask))
-        return normals_release(
-            NormalsArgs<true>{{d_q, scale}, g.width, g.height, g.cell_size, d_normal, d_tan2, d_slope_deg, d_h}, g,
-            slope_lo_deg, slope_hi_deg, d_mask, d_cells, d_n, d_ws, as_stream(stream));
-    st = awo_normals_u16(d_q, g, scale, d_h, d_normal, d_tan2, d_slope_deg, stream);
-    return st != AWO_OK ? st
-                        : awo_release(d_tan2, g, slope_lo_deg, slope_hi_deg, d_mask, d_cells, d_n, d_ws, ws_bytes, stream);
+    return normals_release(
+        NormalsArgs<true>{{d_q, scale}, g.width, g.height, g.cell_size, d_normal, d_tan2, d_slope_deg, d_h}, g,
+        runs_aligned(g, d_q, 8, d_normal, d_tan2, d_slope_deg, d_h, d_mask), slope_lo_deg, slope_hi_deg, d_mask,
+        d_cells, d_n, d_ws, as_stream(stream));
 }
 
 // ---------------------------------------------------------------------------
@@ -1175,8 +1250,7 @@ extern "C" awo_status awo_release_texture(const float* d_tan2, awo_grid g, int32
     auto kern = release_log2 == 0   ? (vec ? k_release_texture_mask<0, true> : k_release_texture_mask<0, false>)
                 : release_log2 == 1 ? (vec ? k_release_texture_mask<1, true> : k_release_texture_mask<1, false>)
                 : release_log2 == 2 ? (vec ? k_release_texture_mask<2, true> : k_release_texture_mask<2, false>)
-                : release_log2 == 3 ? k_release_texture_mask<3, false>
-                                    : k_release_texture_mask<-1, false>;
+                                    : k_release_texture_mask<3, false>;
     if ((release_log2 == 1 || release_log2 == 2) && g.height >= 2 && g.height < 65535 && wr % RT_TILE == 0) {
         // rows are whole tiles: one launch of row groups that share their tan^2 rows
         const dim3 grid((unsigned)(wr / RT_TILE), (unsigned)g.height + 1u);  // at most 65535 groups
@@ -1195,6 +1269,9 @@ extern "C" awo_status awo_release_texture(const float* d_tan2, awo_grid g, int32
                 k_release_texture_rows<2, false><<<grid, RT_THREADS, 0, s>>>(d_tan2, g.width, g.height, (uint32_t)wr,
                                                                             n, scale, t_lo, t_hi, d_mask, tile_count);
         }
+    } else if (release_log2 < 0) {
+        k_release_texture_texels<<<tiles, NC_THREADS, 0, s>>>(d_tan2, g.width, g.height, (uint32_t)wr, (uint32_t)n, scale,
+                                                              t_lo, t_hi, d_mask, tile_count);
     } else {
         kern<<<tiles, RT_THREADS, 0, s>>>(d_tan2, g.width, g.height, (uint32_t)wr, n, scale, t_lo, t_hi, d_mask,
                                           tile_count);

@@ -108,3 +108,48 @@ def test_mask_bytes_of_any_value(size):
     awo.awo_release_from_mask(torch.from_numpy(m).cuda(), g, cells, n, ws)
     torch.cuda.synchronize()
     assert np.array_equal(cells[:int(n)].cpu().numpy(), np.flatnonzero(m))
+
+
+@pytest.mark.parametrize("W,H", [(1, 5000), (3, 3000), (83, 61), (1023, 9), (4097, 3), (4100, 1), (2, 2049), (1799, 1391)])
+@pytest.mark.parametrize("off", [0, 1])
+def test_single_cells_of_any_width_and_offset(W, H, off):
+    """The pass for ragged rows and unaligned buffers, alone and with the release, on values for every form."""
+    dem = _dem(W, H, True)
+    n = W * H
+    nrm, t2, deg = oracle.normals(dem, 10.0)
+    _, cells = oracle.release(t2, 20.0, 60.0)
+    d_h = torch.zeros(n + off, device="cuda")[off:]
+    d_h.copy_(torch.from_numpy(dem.ravel()))
+    g = awo.grid(W, H, 10.0)
+    out = [torch.full((k * n + off,), 7.0, device="cuda")[off:] for k in (3, 1)]
+    awo.awo_normals(d_h, g, out[0], out[1], None)
+    mask = torch.full((n + off,), 9, dtype=torch.uint8, device="cuda")[off:]
+    lst, cnt = torch.zeros(n, dtype=torch.int32, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    ws = torch.empty(awo.awo_release_workspace_bytes(g), dtype=torch.uint8, device="cuda")
+    both = [torch.full((k * n + off,), 7.0, device="cuda")[off:] for k in (3, 1)]
+    awo.awo_terrain(d_h, g, None, d_h, both[0], both[1], None, 20.0, 60.0, mask, lst, cnt, ws)
+    torch.cuda.synchronize()
+    for a, b in (out, both):
+        assert np.array_equal(a.cpu().numpy().view(np.uint32), np.ascontiguousarray(nrm).ravel().view(np.uint32))
+        assert np.array_equal(b.cpu().numpy().view(np.uint32), t2.ravel().view(np.uint32))
+    assert np.array_equal(lst[:int(cnt)].cpu().numpy().view(np.uint32), cells)
+    assert np.array_equal(np.flatnonzero(mask.cpu().numpy()), cells)
+
+
+@pytest.mark.parametrize("r", [-1, -2, -3])
+@pytest.mark.parametrize("W,H", [(8, 8), (17, 700), (1030, 77), (2047, 33)])
+def test_coarse_texture_texels(r, W, H):
+    rng = np.random.default_rng(W * 7 + H)
+    t2 = (rng.random((H, W)) * 2.0).astype(np.float32)
+    t2.ravel()[rng.integers(0, W * H, W * H // 20)] = np.inf
+    t2.ravel()[rng.integers(0, W * H, W * H // 20)] = np.nan
+    g = awo.grid(W, H, 10.0)
+    wr, hr = awo.awo_release_texture_dims(g, r)
+    mask = torch.full((wr * hr,), 9, dtype=torch.uint8, device="cuda")
+    texels, n = torch.zeros(wr * hr, dtype=torch.int32, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    ws = torch.empty(awo.awo_release_texture_workspace_bytes(g, r), dtype=torch.uint8, device="cuda")
+    awo.awo_release_texture(torch.from_numpy(t2).cuda().view(-1), g, r, 30.0, 50.0, mask, texels, n, ws)
+    torch.cuda.synchronize()
+    want_mask, want = oracle.release_texture(t2, r, 30.0, 50.0)
+    assert np.array_equal(mask.cpu().numpy(), np.asarray(want_mask).ravel())
+    assert np.array_equal(texels[:int(n)].cpu().numpy().view(np.uint32), want)
