@@ -144,11 +144,9 @@ awo_status awo_release(const float* d_tan2, awo_grid g, double slope_lo_deg, dou
 
 /*
  * a1 + b, and a0 + a1 + b, in one call: exactly awo_normals followed by
- * awo_release, and awo_normals_u16 followed by awo_release.  Where rows of
- * four cells are 16-byte aligned (width a multiple of 4; heights, normals,
- * tan2 and slope 16-byte, uint16 heights 8-byte, mask 4-byte aligned), tan^2
- * is tested as it is made and not read back.  Arguments, ranges, workspace and
- * errors as in those calls; d_tan2 is required.
+ * awo_release, and awo_normals_u16 followed by awo_release, with tan^2 tested
+ * as it is made and not read back.  Arguments, ranges, workspace and errors as
+ * in those calls; d_tan2 is required.
  */
 awo_status awo_normals_release(const float* d_h, awo_grid g, float* d_normal, float* d_tan2, float* d_slope_deg,
                                double slope_lo_deg, double slope_hi_deg, uint8_t* d_mask, uint32_t* d_cells,

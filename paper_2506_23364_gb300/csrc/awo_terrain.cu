@@ -419,9 +419,8 @@ __global__ void __launch_bounds__(RT_THREADS) k_normals_tiles(const __grid_const
 // The same for any width and alignment: single cells, a warp's side by side,
 // so that every load and store is coalesced whatever the rows' alignment
 // (four consecutive cells a thread, one after the other, touched each sector
-// four times and took 3325 x 4197 with the release pass 238 -> 94 us, 7.7
-// times the aligned kernel's time a cell before and 1.8 now: 3.3 TB/s, bound
-// by issue and by the five loads of a cell).  512 threads: 256 or 1024 took
+// four times and took 3325 x 4197 with the release pass 238 -> 94 us, 4.0
+// times the aligned pass's time a cell before and 1.6 now).  512 threads: 256 or 1024 took
 // 626 x 422 19.1 -> 20-22 us.  A block takes `span` cells: a release tile when
 // it counts one.
 constexpr int NC_THREADS = 512;
