@@ -55,6 +55,9 @@ __global__ void k_finalize(const float* __restrict__ maxe, int64_t n, float g2, 
 // made from the maximum energy as it is needed, vel = sqrt((2 g) maxe), and
 // written (awo_finalize fused in): each level-0 cell is the child of exactly
 // one level-1 texel, so each is computed and written once.
+// Bound by HBM: 8192^2, velocity and a full chain 187 -> 166 us (984 MB, 88% of
+// the copy rate) with 16-byte loads, two level-1 texels a thread and row, where
+// rows are whole groups of four; 8-byte ones for other even rows.
 constexpr int LOD_TILE = 32;   // level-1 tile side
 constexpr int LOD_FUSED = 6;   // levels a block can finish: 32, 16, 8, 4, 2, 1
 
@@ -68,6 +71,7 @@ struct LodArgs {
     float* v[LOD_FUSED];
     int n_out;                               // levels written, 1 .. LOD_FUSED
     bool vec2;                               // level-0 child pairs as uint2 / float2
+    bool vec4;                               // two of them as uint4 / float4, their results as uint2 / float2
 };
 
 template <bool FROM_MAXE>
@@ -91,14 +95,61 @@ __device__ __forceinline__ float2 lod_vel0_pair(const LodArgs& a, uint32_t i)
 }
 
 template <bool FROM_MAXE>
+__device__ __forceinline__ float4 lod_vel0_four(const LodArgs& a, uint32_t i)
+{
+    const float4 x = __ldg(reinterpret_cast<const float4*>(a.v0 + i));
+    if (!FROM_MAXE) return x;
+    const float4 v = make_float4(__fsqrt_rn(__fmul_rn(a.g2, x.x)), __fsqrt_rn(__fmul_rn(a.g2, x.y)),
+                                 __fsqrt_rn(__fmul_rn(a.g2, x.z)), __fsqrt_rn(__fmul_rn(a.g2, x.w)));
+    *reinterpret_cast<float4*>(a.vel0 + i) = v;
+    return v;
+}
+
+__device__ __forceinline__ uint32_t saturated(unsigned long long sum)
+{
+    return sum > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)sum;
+}
+
+template <bool FROM_MAXE>
 __global__ void __launch_bounds__(256) k_lod_fused(const __grid_constant__ LodArgs a)
 {
     __shared__ uint32_t sc[2][LOD_TILE][LOD_TILE + 1];
     __shared__ float sv[2][LOD_TILE][LOD_TILE + 1];
     const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
     const int bx = blockIdx.x, by = blockIdx.y;
-    // level 1 from level 0: four texels per thread, rows ty, ty + 8, ...
-    {
+    // level 1 from level 0
+    if (a.vec4) {  // two texels a thread and row: w0 a multiple of 4, so both exist or neither
+        const int w0 = a.w[0], h0 = a.h[0], w1 = a.w[1], h1 = a.h[1];
+        const int x = 2 * (tid & 15), X = bx * LOD_TILE + x;
+#pragma unroll
+        for (int k = 0; k < LOD_TILE / 16; ++k) {
+            const int y = (tid >> 4) + 16 * k, Y = by * LOD_TILE + y;
+            if (X < w1 && Y < h1) {
+                const uint32_t r0 = (uint32_t)(2 * Y) * (uint32_t)w0 + (uint32_t)(2 * X);
+                const uint4 c_0 = __ldg(reinterpret_cast<const uint4*>(a.c0 + r0));
+                const float4 v_0 = lod_vel0_four<FROM_MAXE>(a, r0);
+                unsigned long long sl = (unsigned long long)c_0.x + c_0.y, sr = (unsigned long long)c_0.z + c_0.w;
+                float ml = fmaxf(v_0.x, v_0.y), mr = fmaxf(v_0.z, v_0.w);
+                if (2 * Y + 1 < h0) {
+                    const uint32_t r1 = r0 + (uint32_t)w0;
+                    const uint4 c_1 = __ldg(reinterpret_cast<const uint4*>(a.c0 + r1));
+                    const float4 v_1 = lod_vel0_four<FROM_MAXE>(a, r1);
+                    sl += (unsigned long long)c_1.x + c_1.y;
+                    sr += (unsigned long long)c_1.z + c_1.w;
+                    ml = fmaxf(ml, fmaxf(v_1.x, v_1.y));
+                    mr = fmaxf(mr, fmaxf(v_1.z, v_1.w));
+                }
+                const uint2 c = make_uint2(saturated(sl), saturated(sr));
+                const uint32_t o = (uint32_t)Y * (uint32_t)w1 + (uint32_t)X;  // even: w1 and X are
+                *reinterpret_cast<uint2*>(a.c[0] + o) = c;
+                *reinterpret_cast<float2*>(a.v[0] + o) = make_float2(ml, mr);
+                sc[0][y][x] = c.x;
+                sc[0][y][x + 1] = c.y;
+                sv[0][y][x] = ml;
+                sv[0][y][x + 1] = mr;
+            }
+        }
+    } else {  // four texels per thread, rows ty, ty + 8, ...
         const int w0 = a.w[0], h0 = a.h[0], w1 = a.w[1], h1 = a.h[1];
         const int X = bx * LOD_TILE + tx;
 #pragma unroll
@@ -137,7 +188,7 @@ __global__ void __launch_bounds__(256) k_lod_fused(const __grid_constant__ LodAr
                         }
                     }
                 }
-                const uint32_t c = sum > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)sum;
+                const uint32_t c = saturated(sum);
                 const uint32_t o = (uint32_t)Y * (uint32_t)w1 + (uint32_t)X;
                 a.c[0][o] = c;
                 a.v[0][o] = m;
@@ -171,7 +222,7 @@ __global__ void __launch_bounds__(256) k_lod_fused(const __grid_constant__ LodAr
                         m = fmaxf(m, sv[src][2 * y + 1][2 * x + 1]);
                     }
                 }
-                const uint32_t c = sum > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)sum;
+                const uint32_t c = saturated(sum);
                 const uint32_t o = (uint32_t)Y * (uint32_t)a.w[l] + (uint32_t)X;
                 a.c[l - 1][o] = c;
                 a.v[l - 1][o] = m;
@@ -226,6 +277,9 @@ static awo_status lod_levels(const uint32_t* d_count, const float* v0, bool from
         }
         a.vec2 = w % 2 == 0 &&
                  ((((uintptr_t)a.c0) | ((uintptr_t)a.v0) | (from_maxe ? (uintptr_t)d_vel : (uintptr_t)0)) & 7u) == 0;
+        a.vec4 = w % 4 == 0 &&
+                 ((((uintptr_t)a.c0) | ((uintptr_t)a.v0) | (from_maxe ? (uintptr_t)d_vel : (uintptr_t)0)) & 15u) == 0 &&
+                 ((((uintptr_t)a.c[0]) | ((uintptr_t)a.v[0])) & 7u) == 0;
         const dim3 grid((unsigned)((a.w[1] + LOD_TILE - 1) / LOD_TILE), (unsigned)((a.h[1] + LOD_TILE - 1) / LOD_TILE));
         if (from_maxe)
             k_lod_fused<true><<<grid, 256, 0, s>>>(a);

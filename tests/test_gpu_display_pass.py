@@ -49,3 +49,37 @@ def test_snow_unaligned_inputs(W, H, off_h, off_nz):
     want_a, want_rgba = oracle.snow_cover(h, nz, 1500.0, 300.0, 36.0, 4.0)
     assert np.array_equal(alpha.cpu().numpy(), np.asarray(want_a).reshape(H, W))
     assert np.array_equal(rgba.cpu().numpy(), np.asarray(want_rgba).reshape(H, W, 4))
+
+
+@pytest.mark.parametrize("in_place", [False, True])
+@pytest.mark.parametrize("off_in,off_out", [(0, 0), (2, 0), (1, 0), (0, 1), (0, 2)])
+@pytest.mark.parametrize("W,H", [(4, 1), (4, 130), (68, 5), (132, 33), (66, 7), (67, 64), (128, 65)])
+def test_mipmap_widths_and_alignments(W, H, off_in, off_out, in_place):
+    """Rows of whole groups of four, of pairs and odd ones; inputs and level 1 off 16 and 8 bytes."""
+    n, levels = W * H, 4
+    rng = np.random.default_rng(n + off_in)
+    count = rng.integers(0, 2 ** 32, (H, W), dtype=np.uint64).astype(np.uint32)
+    count[rng.random((H, W)) < 0.7] = 5
+    maxe = (rng.random((H, W)) * 400).astype(np.float32)
+    g = awo.grid(W, H, 10.0)
+
+    def buf(size, dtype, off):
+        return torch.zeros(size + off, dtype=dtype, device="cuda")[off:]
+
+    c0, e0 = buf(n, torch.int32, off_in), buf(n, torch.float32, off_in)
+    c0.copy_(torch.from_numpy(count.view(np.int32).ravel()))
+    e0.copy_(torch.from_numpy(maxe.ravel()))
+    vel = e0 if in_place else buf(n, torch.float32, off_in)
+    sizes = [a * b for a, b in awo.lod_shapes(g, levels)[1:]]
+    cl = [buf(s, torch.int32, off_out) for s in sizes]
+    vl = [buf(s, torch.float32, off_out) for s in sizes]
+    awo.awo_finalize_lod(e0, c0, g, 9.81, levels, vel, cl, vl)
+    want_vel = oracle.finalize(maxe, 9.81)
+    want_c, want_v = oracle.lod(count, want_vel, levels)
+    assert np.array_equal(vel.cpu().numpy(), want_vel.ravel())
+    cl2, vl2 = [torch.zeros_like(t) for t in cl], [torch.zeros_like(t) for t in vl]
+    awo.awo_overlay_lod(c0, vel, g, levels, cl2, vl2)
+    for l in range(1, levels):
+        for c, v in ((cl, vl), (cl2, vl2)):
+            assert np.array_equal(c[l - 1].cpu().numpy().view(np.uint32), want_c[l].ravel()), l
+            assert np.array_equal(v[l - 1].cpu().numpy(), want_v[l].ravel()), l
