@@ -130,7 +130,7 @@ __device__ __forceinline__ float4 load4(const float* __restrict__ p, int64_t q, 
 // tail.  The inputs need not be: the third plane of normals whose cell count
 // is not a multiple of 4 starts off a 16-byte boundary, and the four loads of
 // a thread then share its neighbours' sectors in the L1.  Bound by HBM:
-// 5003 x 4099 with such a plane 86 -> 62 us.
+// 5003 x 4099 with such a plane 86 -> 62 us, with the larger grid (below) 53.
 template <bool ALIGNED>
 __global__ void __launch_bounds__(256, 8) k_snow(const float* __restrict__ h, const float* __restrict__ nz, int64_t n,
                                                  float a0, float a1, float c0, float c1, float* __restrict__ alpha,
@@ -211,7 +211,11 @@ extern "C" awo_status awo_snow_cover(const float* d_h, const float* d_nz, awo_gr
     const bool vec4 = ((((uintptr_t)d_alpha) | ((uintptr_t)d_rgba)) & 15u) == 0;
     const bool vec_h = (((uintptr_t)d_h) & 15u) == 0, vec_nz = (((uintptr_t)d_nz) & 15u) == 0;
     auto kern = vec_h && vec_nz ? k_snow<true> : k_snow<false>;
-    kern<<<stream_blocks(vec4 ? n / 4 + 1 : n, 256), 256, 0, as_stream(stream)>>>(d_h, d_nz, n, a0, a1, c0, c1, d_alpha,
-                                                                                  d_rgba, vec4, vec_h, vec_nz);
+    // up to 64 blocks an SM, a group or two a thread: with 8, whose threads loop
+    // and wait for each group's loads in turn, 5003 x 4099 took 62.5 us (16: 59.6,
+    // 32: 54.2, 64: 52.5, a block for every 256 groups 52.6), 6144^2 109.6 (91.9 with
+    // 64), 2048^2 the same 12.2
+    kern<<<stream_blocks(vec4 ? n / 4 + 1 : n, 256, 64), 256, 0, as_stream(stream)>>>(
+        d_h, d_nz, n, a0, a1, c0, c1, d_alpha, d_rgba, vec4, vec_h, vec_nz);
     return launch_status();
 }
