@@ -83,3 +83,33 @@ def test_mipmap_widths_and_alignments(W, H, off_in, off_out, in_place):
         for c, v in ((cl, vl), (cl2, vl2)):
             assert np.array_equal(c[l - 1].cpu().numpy().view(np.uint32), want_c[l].ravel()), l
             assert np.array_equal(v[l - 1].cpu().numpy(), want_v[l].ravel()), l
+
+
+@pytest.mark.parametrize("hit", [0.0, 0.02, 0.5, 1.0])
+@pytest.mark.parametrize("count_min,alpha", [(0, 0.7), (1, 0.7), (1, 0.0), (3, 1.0), (2 ** 32 - 1, 0.5)])
+@pytest.mark.parametrize("n_stops", [2, 5, 16])
+def test_compose_groups_without_hits(n_stops, count_min, alpha, hit):
+    """Groups below count_min, among hit ones and alone, over a base and in place of it; several groups a thread."""
+    W, H = 1283, 977  # more groups than one sweep of the smallest grid, and a tail
+    rng = np.random.default_rng(n_stops + int(100 * hit))
+    value = (rng.random((H, W)) * 80 - 10).astype(np.float32)
+    at = rng.integers(0, W * H, 2000)
+    value.ravel()[at] = np.array([np.nan, np.inf, -np.inf, -0.0], np.float32)[at % 4]
+    count = rng.integers(0, 6, (H, W)).astype(np.uint32)
+    count[np.repeat(rng.random(W * H // 7 + 1), 7)[:W * H].reshape(H, W) >= hit] = 0  # runs that straddle groups
+    base = rng.integers(0, 256, (H, W, 4)).astype(np.uint8)
+    x = np.linspace(0.0, 60.0, n_stops)
+    stops = [(float(x[k]), tuple(int(c) for c in rng.integers(0, 256, 3))) for k in range(n_stops)]
+    cm = awo.Colormap.make(stops, alpha=alpha, count_min=count_min)
+    g = awo.grid(W, H, 10.0)
+    v, c = torch.from_numpy(value).cuda(), torch.from_numpy(count.view(np.int32)).cuda()
+    b = torch.from_numpy(base).cuda()
+    out = torch.empty_like(b)
+    awo.awo_compose(v, c, g, cm, b, out)
+    bare = torch.empty_like(b)
+    awo.awo_compose(v, c, g, cm, None, bare)
+    awo.awo_compose(v, c, g, cm, b, b)
+    want = oracle.compose(value, count, stops, alpha, count_min, base)
+    assert np.array_equal(out.cpu().numpy(), want)
+    assert np.array_equal(b.cpu().numpy(), want)
+    assert np.array_equal(bare.cpu().numpy(), oracle.compose(value, count, stops, alpha, count_min))
