@@ -342,8 +342,8 @@ typedef struct {
 /* Launch shape of the batched particle kernel (the autotuner's search space).
  *   threads_per_block: 64, 128 or 256 (0 = 128)
  *   group_particles:   particles a warp takes per fetch, 32 .. 65536 (0 = chosen
- *                      per request: about its particles / (16 x the launch's
- *                      warps), rounded down to a multiple of 32, within 32 .. 1024)
+ *                      from the particles and the launch's warps, a multiple of
+ *                      32 within 32 .. 1024)
  *   refill: AWO_REFILL_LANE -- lanes whose particle has ended take another one
  *           while the warp's other lanes keep moving (trajectory per thread,
  *           continuously refilled);

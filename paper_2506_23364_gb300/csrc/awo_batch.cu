@@ -4,28 +4,25 @@
 // request table travels in the kernels' parameter blocks, so a call needs no
 // host-to-device copy and can be captured in a CUDA graph.  Kernels:
 //   k_batch_prepare  one block: release counts (possibly on the device), the
-//                    prefix sums of cells, zeroed counters;
+//                    prefix sums of cells and of units of work, zeroed
+//                    counters;
 //   k_batch_starts   per release cell of every request: its start record (in
 //                    the processing order of awo_particle.cuh) and
 //                    the release visits of its particles;
-//   k_simulate       one launch per request (awo_simulate.cu), each allowed to
-//                    start while the one before it still runs its last
-//                    particles, so that the requests run as one stream of
-//                    work without a tail between them.  A request's
-//                    constants are then at fixed places of the parameter
-//                    block: one persistent kernel over all requests kept them
-//                    in registers (62 of them, 90 with the pool: 5 blocks an
-//                    SM), and read by request index they cost 21 of 189 warp
-//                    instructions per move.  12 regions 512^2..2048^2, the
-//                    particle part: 9.71 ms as one kernel, 8.23 ms so.
+//   k_simulate       for a request with many particles, a launch of its own
+//                    (awo_simulate.cu), allowed to start while the one before
+//                    it still runs its last particles;
+//   k_batch_simulate for all others together, persistent: a warp takes a unit,
+//                    which names a request, and runs that request's particles
+//                    (run_particles, the loop of awo_simulate) until none is
+//                    left to take.
 // Every request's rasters equal those of awo_simulate on that request alone:
-// it is the same kernel.
+// the particles take the same steps.
 #include <math.h>
 
 #include <algorithm>
 #include <cstddef>
 #include <cstring>
-#include <mutex>
 #include <vector>
 
 #include "awo_particle.cuh"
@@ -43,15 +40,28 @@ struct BatchReq {
     const uint32_t* n_cells_dev;
     uint32_t n_cells_max, n_grid, N;
     uint32_t starts_off;  // its first 32-byte start-record slot
+    uint32_t id;          // its index in the caller's array
+    uint32_t own_launch;  // OwnLaunch
     TexelGeom tg;
 };
 
+// Requests that share an instance of the particle kernel: records of texels
+// or cells, footprints by texture or by loads.
+constexpr int BATCH_KINDS = 2;
+
+// Requests are in launch order (BatchArgs.r) but for the statistics of ws,
+// which are in the caller's.
 struct BatchHeader {
-    SimWorkspace ws[AWO_BATCH_MAX];           // each request's work counter (and statistics)
-    uint32_t cell_prefix[AWO_BATCH_MAX + 1];  // start records before each request
+    SimWorkspace ws[AWO_BATCH_MAX];            // work counters (and statistics)
+    unsigned long long n_part[AWO_BATCH_MAX];  // particles of each request for k_batch_simulate
+    uint32_t cell_prefix[AWO_BATCH_MAX + 1];   // start records before each request
+    uint32_t unit_prefix[AWO_BATCH_MAX + 1];   // units of work before each request
     uint32_t n_cells[AWO_BATCH_MAX];
-    uint32_t check;                           // check_pays of the whole batch
-    uint32_t order_sinv[AWO_BATCH_MAX];       // processing order of each request's entries
+    uint32_t own_cells[AWO_BATCH_MAX];   // n_cells of the requests with a launch of their own, else 0
+    uint32_t order_sinv[AWO_BATCH_MAX];  // processing order of each request's entries
+    uint32_t next_unit[BATCH_KINDS];     // units taken, by launch
+    uint32_t chunk;                      // particles a warp takes per fetch, at most
+    uint32_t check;                      // check_pays of the whole batch
 };
 constexpr size_t BATCH_HEADER_BYTES = ((sizeof(BatchHeader) + 255) / 256) * 256;
 
@@ -62,6 +72,7 @@ static_assert(sizeof(awo_tuning) == 16, "awo_tuning layout (C ABI)");
 struct BatchArgs {
     BatchReq r[AWO_BATCH_MAX];
     uint32_t n_req;
+    uint32_t sim_warps;           // warps of k_batch_simulate's launch
     unsigned long long look_min;  // look_paths of whole-cell steps
     BatchHeader* hdr;
     unsigned long long* stats;  // 6 per request, stats_step words apart
@@ -69,6 +80,62 @@ struct BatchArgs {
     TexelStart* starts;  // one 32-byte slot per release-list entry (CellStarts fill the first half of a request's)
 };
 static_assert(sizeof(BatchArgs) <= 32764, "the request table must fit the kernel parameter block");
+
+// A request of the particle kernel (names read by AWO_MOVE_WORDS and run_particles, as in SimArgs).
+struct BatchSimReq {
+    const float* h;
+    uint32_t* count;
+    float* maxe;
+    int W, H;
+    float Wm1, Hm1, P, oneP, R, s, R23, kD, muD;
+    uint32_t max_steps;
+    KeysTable keys;
+    uint32_t N, id;
+    void* starts;
+    cudaTextureObject_t tex;
+};
+
+struct BatchSimArgs {
+    BatchSimReq r[AWO_BATCH_MAX];
+    uint32_t first, n;   // the launch's requests
+    uint32_t kind;       // its work counter
+    uint32_t group;      // particles a warp takes per fetch, 0: chosen by the kernel
+    uint32_t min_idle;   // idle lanes a refill needs: 1, or 32 (lock-step batches)
+    BatchHeader* hdr;
+    unsigned long long* stats;
+    uint32_t stats_step;
+};
+static_assert(sizeof(BatchSimArgs) <= 32764, "the request table must fit the kernel parameter block");
+
+// How the particles of a batch are shared out.  A unit of work stands for one
+// warp on one request: the warp that takes it runs the request's particles
+// until none is left to take.  The batch has UNITS_PER_WARP units for each
+// warp of the launch, split over the requests by their particles, so that
+// some requests are always at work while another one's last particles run
+// out; but the warps of an SM that work on many requests keep pushing one
+// another's constants out of the constant cache, so a request gets at least
+// one in REQUESTS_IN_FLIGHT of the warps (or one for every 32 of its
+// particles).  A warp that finds no unit left joins a request that has more
+// particles waiting than its own warps take next.  Measured (ms; 128 regions
+// of 256^2 with 64 particles per release cell / 32 of 1024^2 with 32): 1 unit a
+// warp and no least share 7.0 / 8.6, 2 and the share of 1 in 8 2.77 / 3.84, all
+// warps on every request in turn 4.0 / 5.8.
+constexpr uint32_t UNITS_PER_WARP = 2, REQUESTS_IN_FLIGHT = 8;
+constexpr uint32_t CHUNKS_PER_WARP = 32;  // fetches a warp makes on an even split (16: 12 of 1280^2 5.80 -> 5.95 ms)
+
+// Requests with a launch of k_simulate each: their constants are then at
+// fixed places of the parameter block, which runs up to 167 G moves/s where
+// k_batch_simulate, issue-bound, ends at 140; but a launch leaves the GPU
+// partly idle at its end, and costs the host 7 us.  4 regions of 2048^2: 24 M
+// particles each 6.02 against 7.36 ms, 6 M each 2.80 against 2.10; 12 of 1280^2,
+// 5.9 M each, 7.7 against 5.8; 12 of 512^2..2048^2 7.97 with the line at 6 M, 8.14
+// at 10 M, 8.47 without launches of their own (7.75 with one for each).  The
+// number of particles is known on the device alone, so the host launches for
+// every request that can have LARGE_PARTICLES at the share of release cells
+// that steep terrain has (1 in 22), and the launch ends at once when there are
+// fewer.  A request that is alone of its kind has its own launch, too.
+constexpr unsigned long long LARGE_PARTICLES = 6000000ull, LARGE_MOST = 22ull * LARGE_PARTICLES;
+enum OwnLaunch : uint32_t { OWN_NEVER, OWN_IF_LARGE, OWN_ALWAYS };
 
 // Index r with prefix[r] <= g < prefix[r+1] (prefix has n + 1 entries).
 template <typename T>
@@ -85,42 +152,79 @@ __device__ __forceinline__ int find_request(const T* prefix, int n, T g)
     return lo;
 }
 
+// Sum over the lanes of a warp up to this one.
+template <typename T>
+__device__ __forceinline__ T warp_inclusive(T v)
+{
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const T t = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += t;
+    }
+    return v;
+}
+
+// One thread per request.
 __global__ void __launch_bounds__(AWO_BATCH_MAX) k_batch_prepare(const __grid_constant__ BatchArgs a)
 {
-    __shared__ uint32_t s_nc[AWO_BATCH_MAX];
-    __shared__ unsigned long long s_np[AWO_BATCH_MAX];
-    const int t = threadIdx.x;
+    constexpr int WARPS = AWO_BATCH_MAX / 32;
+    __shared__ unsigned long long s_total[WARPS], s_grid[WARPS];
+    __shared__ double s_paths[WARPS];
+    __shared__ uint32_t s_cells[WARPS], s_units[WARPS];
+    const int t = threadIdx.x, warp = t >> 5;
+    const bool last_lane = (t & 31) == 31;
+    const bool mine = t < (int)a.n_req;
     uint32_t nc = 0u;
-    if (t < (int)a.n_req) {
+    unsigned long long np = 0ull, grid = 0ull;
+    double paths = 0.0;  // particles over their steps, as in look_paths
+    if (mine) {
         const BatchReq& q = a.r[t];
         nc = q.n_cells_max;
         if (q.n_cells_dev) nc = min(nc, *q.n_cells_dev);
         if (q.N == 0u) nc = 0u;  // no particles, no release visits
         a.hdr->n_cells[t] = nc;
         a.hdr->order_sinv[t] = order_stride_inverse(nc / order_block(q.N));
-    }
-    s_nc[t] = nc;
-    // particles for the particle kernel: none for a request with max_steps = 0
-    // (every particle capped at its release visit, counted by k_batch_starts)
-    s_np[t] = (t < (int)a.n_req && a.r[t].max_steps != 0u) ? (unsigned long long)nc * a.r[t].N : 0ull;
-    if (t < (int)a.n_req) {
+        // particles for the particle kernel: none for a request with max_steps = 0
+        // (every particle capped at its release visit, counted by k_batch_starts)
+        np = q.max_steps != 0u ? (unsigned long long)nc * q.N : 0ull;
+        grid = q.n_grid;
+        paths = (double)np / q.s;
         a.hdr->ws[t] = SimWorkspace{};
         for (int i = 0; i < 6; ++i) a.stats[(size_t)t * a.stats_step + i] = 0ull;
     }
+    const unsigned long long np_up = warp_inclusive(np), grid_up = warp_inclusive(grid);
+    const double paths_up = warp_inclusive(paths);
+    if (last_lane) s_total[warp] = np_up, s_grid[warp] = grid_up, s_paths[warp] = paths_up;
     __syncthreads();
+    unsigned long long total = 0ull;
+#pragma unroll
+    for (int w = 0; w < WARPS; ++w) total += s_total[w];
+    const bool own = mine && (a.r[t].own_launch == OWN_ALWAYS ||
+                              (a.r[t].own_launch == OWN_IF_LARGE && np >= LARGE_PARTICLES));
+    // FP32 is enough to share out the work (a 64-bit division costs more than the rest of this kernel)
+    const float warps = (float)a.sim_warps, unit = fmaxf((float)total / (warps * UNITS_PER_WARP), 32.0f);
+    const float least = fminf((float)np / 32.0f, warps / REQUESTS_IN_FLIGHT);
+    const uint32_t units = own ? 0u : (uint32_t)ceilf(fminf(fmaxf((float)np / unit, least), warps));
+    uint32_t cells1 = warp_inclusive(nc), units1 = warp_inclusive(units);
+    if (last_lane) s_cells[warp] = cells1, s_units[warp] = units1;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < WARPS; ++w)
+        if (w < warp) cells1 += s_cells[w], units1 += s_units[w];
+    if (t < BATCH_KINDS) a.hdr->next_unit[t] = 0u;
+    a.hdr->n_part[t] = own ? 0ull : np;
+    a.hdr->own_cells[t] = own ? nc : 0u;
+    a.hdr->cell_prefix[t + 1] = cells1;
+    a.hdr->unit_prefix[t + 1] = units1;
     if (t == 0) {
-        unsigned long long total = 0ull, grid = 0ull;
-        double paths = 0.0;  // particles over their steps, as in look_paths
-        uint32_t cs = 0u;
-        for (int r = 0; r < (int)a.n_req; ++r) {
-            a.hdr->cell_prefix[r] = cs;
-            cs += s_nc[r];
-            total += s_np[r];
-            paths += (double)s_np[r] / a.r[r].s;
-            grid += a.r[r].n_grid;
-        }
-        a.hdr->cell_prefix[a.n_req] = cs;
-        a.hdr->check = paths >= (double)a.look_min || total >= 7ull * grid ? 1u : 0u;  // as check_pays
+        a.hdr->cell_prefix[0] = a.hdr->unit_prefix[0] = 0u;
+        unsigned long long grids = 0ull;
+        double sum_paths = 0.0;
+#pragma unroll
+        for (int w = 0; w < WARPS; ++w) grids += s_grid[w], sum_paths += s_paths[w];
+        a.hdr->chunk = max((uint32_t)fminf((float)total / (warps * CHUNKS_PER_WARP), 1024.0f) & ~31u, 32u);
+        a.hdr->check = sum_paths >= (double)a.look_min || total >= 7ull * grids ? 1u : 0u;  // as check_pays
     }
 }
 
@@ -154,13 +258,92 @@ __global__ void __launch_bounds__(256) k_batch_starts(const __grid_constant__ Ba
         }
         // particles of entries outside the grid are rejected; with max_steps = 0
         // every particle is capped at its release visit (no particle kernel work)
-        unsigned long long* st6 = a.stats + (size_t)r * a.stats_step;
+        unsigned long long* st6 = a.stats + (size_t)q.id * a.stats_step;
         if (!ok) atomicAdd(st6 + 5, (unsigned long long)q.N);
         if (ok && q.max_steps == 0u) {
             atomicAdd(st6 + 1, (unsigned long long)q.N);
             atomicAdd(st6 + 3, (unsigned long long)q.N);
         }
     }
+}
+
+// One launch per kind of request and instance (with and without the look: one
+// of the two ends at once, as in k_simulate).  Persistent; the last block
+// orders the launch after the one before it (see k_simulate).
+//
+// A request's constants are read from the parameter block through an index
+// that the compiler knows to be the same for the whole warp (it comes from
+// ballots): held in a lane's registers they took 62-92 of them.  64 registers,
+// 8 blocks an SM: 48 (and 16 bytes spilled) gave 2% more on large requests and
+// took 5-8% longer on small ones, which are bound by latency.  128 regions of
+// 64^2 1.44 -> 0.85 ms against a launch for each, of 512^2 with 16 particles per
+// release cell 5.43 -> 2.85, 32 of 1024^2 with 32 6.05 -> 3.84.
+template <bool TEXELS, bool PLAIN, bool CHECK>
+__global__ void __launch_bounds__(256, 4) k_batch_simulate(const __grid_constant__ BatchSimArgs a)
+{
+    extern __shared__ uint32_t s_pool[];  // POOL_WORDS per warp
+    asm volatile("griddepcontrol.launch_dependents;");
+    if (blockIdx.x == gridDim.x - 1u) {
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        return;
+    }
+    if ((a.hdr->check != 0u) != CHECK) return;
+    const uint32_t lane = threadIdx.x & 31u;
+    uint32_t* pool = s_pool + (threadIdx.x >> 5) * POOL_WORDS;
+    const uint32_t* prefix = a.hdr->unit_prefix + a.first;
+    bool units_left = true;
+    while (true) {
+        uint32_t g = 0u, i = 0u;
+        if (units_left) {
+            if (lane == 0u) g = atomicAdd(&a.hdr->next_unit[a.kind], 1u);
+            g = prefix[0] + __shfl_sync(0xffffffffu, g, 0);
+            units_left = g < prefix[a.n];
+        }
+        if (units_left) {
+            // the request of unit g: as many come before it as end at or below g
+#pragma unroll
+            for (uint32_t k = 0u; k < AWO_BATCH_MAX; k += 32u)
+                i += (uint32_t)__popc(__ballot_sync(0xffffffffu, k + lane < a.n && prefix[k + lane + 1u] <= g));
+        } else {
+            // no unit left: the first request with more particles waiting than its own warps take next
+            i = a.n;
+            for (uint32_t k = 0u; k < a.n && i == a.n; k += 32u) {
+                const uint32_t j = min(k + lane, a.n - 1u), c = a.first + j;
+                const unsigned which =
+                    __ballot_sync(0xffffffffu, __ldcg(&a.hdr->ws[c].next_item) + 32ull * (prefix[j + 1u] - prefix[j]) <
+                                                   a.hdr->n_part[c]);
+                if (which) i = min(k + (uint32_t)__ffs(which) - 1u, a.n - 1u);
+            }
+            if (i == a.n) break;
+        }
+        const uint32_t r = a.first + i;
+        const BatchSimReq& q = a.r[r];
+        const unsigned long long total = a.hdr->n_part[r];
+        unsigned long long* stats = a.stats + (size_t)q.id * a.stats_step;
+        const uint32_t unit0 = prefix[i], units = prefix[i + 1] - unit0;
+        if (units_left && g == unit0 && lane == 0u) {
+            // particles of entries inside the grid (the prologue has counted the others)
+            const unsigned long long run = total - stats[5];
+            stats[1] = run;
+            atomicAdd(&stats[4], run);
+        }
+        // particles a warp takes per fetch: the batch's, or one warp's share where that is less
+        const unsigned long long share = total / units;
+        uint32_t chunk = share < a.hdr->chunk ? max((uint32_t)share & ~31u, 32u) : a.hdr->chunk;
+        if (a.group) chunk = a.group;
+        if (q.tex)
+            run_particles<TEXELS, 1, CHECK, PLAIN>(q, total, chunk, a.min_idle, &a.hdr->ws[r].next_item, stats, pool);
+        else
+            run_particles<TEXELS, 0, CHECK, PLAIN>(q, total, chunk, a.min_idle, &a.hdr->ws[r].next_item, stats, pool);
+        __syncwarp();  // the pool is empty; its words before the next request's
+    }
+}
+
+template <bool TEXELS, bool PLAIN>
+static awo_status launch_kind(const BatchSimArgs& a, int threads, bool early, cudaStream_t s)
+{
+    const awo_status st = launch_persistent<k_batch_simulate<TEXELS, PLAIN, true>>(a, threads, early, s);
+    return st != AWO_OK ? st : launch_persistent<k_batch_simulate<TEXELS, PLAIN, false>>(a, threads, true, s);
 }
 
 static bool tuning_ok(const awo_tuning* t)
@@ -210,8 +393,6 @@ extern "C" awo_status awo_simulate_batched(const awo_sim_request* reqs, int32_t 
     if ((((uintptr_t)d_ws) & 15u) != 0) return AWO_EINVAL;
     if (ws_bytes < BATCH_HEADER_BYTES + (size_t)total * sizeof(TexelStart)) return AWO_ENOMEM;
     const int threads = (tuning && tuning->threads_per_block) ? tuning->threads_per_block : 128;
-    const uint32_t group = tuning ? (uint32_t)tuning->group_particles : 0u;
-    const int refill = tuning ? tuning->refill : AWO_REFILL_LANE;
     cudaStream_t s = as_stream(stream);
 
     BatchArgs a;
@@ -224,50 +405,104 @@ extern "C" awo_status awo_simulate_batched(const awo_sim_request* reqs, int32_t 
     const bool direct = d_stats && (((uintptr_t)d_stats) & 7u) == 0;
     a.stats = direct ? reinterpret_cast<unsigned long long*>(d_stats) : a.hdr->ws[0].stats;
     a.stats_step = (uint32_t)((direct ? sizeof(awo_sim_stats) : sizeof(SimWorkspace)) / sizeof(unsigned long long));
-    SimArgs sim[AWO_BATCH_MAX];  // (no allocation that could throw)
-    uint32_t off = 0;
-    for (int i = 0; i < n_req; ++i) {
-        const awo_sim_request& q = reqs[i];
-        SimArgs& c = sim[i];
-        sim_constants(c, q.d_h, q.grid, &q.params, q.d_count, q.d_maxe, s);
-        c.n_cells_dev = a.hdr->n_cells + i;
-        c.n_cells_max = q.n_cells_max;
-        c.next_item = &a.hdr->ws[i].next_item;
-        c.stats = a.stats + (size_t)i * a.stats_step;
-        c.starts = a.starts + off;
-        c.group = group;
-        c.min_idle = refill == AWO_REFILL_WARP ? 32u : 1u;
-        c.check = &a.hdr->check;
-        BatchReq& b = a.r[i];
-        b.h = q.d_h;
-        b.count = q.d_count;
-        b.W = c.W;
-        b.H = c.H;
-        b.P = c.P;
-        b.oneP = c.oneP;
-        b.s = c.s;
-        b.max_steps = c.max_steps;
-        b.cells = q.d_cells;
-        b.n_cells_dev = q.d_n_cells;
-        b.n_cells_max = q.n_cells_max;
-        b.n_grid = c.n_grid;
-        b.N = c.N;
-        b.starts_off = off;
-        b.tg = c.tg;
-        off += q.n_cells_max;
-        if (q.params.flags & AWO_SIM_CLEAR_OUTPUTS) {
-            const size_t bytes = (size_t)cells_of(q.grid) * sizeof(uint32_t);
-            if (cudaMemsetAsync(q.d_count, 0, bytes, s) != cudaSuccess) return AWO_ECUDA;
-            if (cudaMemsetAsync(q.d_maxe, 0, bytes, s) != cudaSuccess) return AWO_ECUDA;
+    // the requests by kind, each kind's in the caller's order
+    BatchSimArgs b;
+    memset(&b, 0, sizeof(b));
+    b.hdr = a.hdr;
+    b.stats = a.stats;
+    b.stats_step = a.stats_step;
+    b.group = tuning ? (uint32_t)tuning->group_particles : 0u;
+    b.min_idle = tuning && tuning->refill == AWO_REFILL_WARP ? 32u : 1u;
+    bool plain = true;
+    uint32_t kind_first[BATCH_KINDS + 1] = {0}, off = 0, at = 0;
+    SimArgs own[AWO_BATCH_MAX];
+    for (int kind = 0; kind < BATCH_KINDS; ++kind) {
+        kind_first[kind] = at;
+        for (int i = 0; i < n_req; ++i) {
+            if ((reqs[i].params.release_log2 != 0) != (kind == 1)) continue;
+            const awo_sim_request& q = reqs[i];
+            SimArgs& c = own[at];
+            sim_constants(c, q.d_h, q.grid, &q.params, q.d_count, q.d_maxe, s);
+            BatchSimReq& d = b.r[at];
+            d.h = c.h;
+            d.count = c.count;
+            d.maxe = c.maxe;
+            d.W = c.W;
+            d.H = c.H;
+            d.Wm1 = c.Wm1;
+            d.Hm1 = c.Hm1;
+            d.P = c.P;
+            d.oneP = c.oneP;
+            d.R = c.R;
+            d.s = c.s;
+            d.R23 = c.R23;
+            d.kD = c.kD;
+            d.muD = c.muD;
+            d.max_steps = c.max_steps;
+            d.keys = c.keys;
+            d.N = c.N;
+            d.id = (uint32_t)i;
+            d.starts = a.starts + off;
+            d.tex = c.tex;
+            plain = plain && c.s == 1.0f && c.kD == 0.0f;
+            BatchReq& e = a.r[at];
+            e.h = c.h;
+            e.count = c.count;
+            e.W = c.W;
+            e.H = c.H;
+            e.P = c.P;
+            e.oneP = c.oneP;
+            e.s = c.s;
+            e.max_steps = c.max_steps;
+            e.cells = q.d_cells;
+            e.n_cells_dev = q.d_n_cells;
+            e.n_cells_max = q.n_cells_max;
+            e.n_grid = c.n_grid;
+            e.N = c.N;
+            e.starts_off = off;
+            e.id = (uint32_t)i;
+            e.own_launch = (unsigned long long)q.n_cells_max * c.N >= LARGE_MOST ? OWN_IF_LARGE : OWN_NEVER;
+            e.tg = c.tg;
+            off += q.n_cells_max;
+            ++at;
+            if (q.params.flags & AWO_SIM_CLEAR_OUTPUTS) {
+                const size_t bytes = (size_t)cells_of(q.grid) * sizeof(uint32_t);
+                if (cudaMemsetAsync(q.d_count, 0, bytes, s) != cudaSuccess) return AWO_ECUDA;
+                if (cudaMemsetAsync(q.d_maxe, 0, bytes, s) != cudaSuccess) return AWO_ECUDA;
+            }
         }
     }
+    kind_first[BATCH_KINDS] = at;
+    for (int kind = 0; kind < BATCH_KINDS; ++kind)
+        if (kind_first[kind + 1] == kind_first[kind] + 1u) a.r[kind_first[kind]].own_launch = OWN_ALWAYS;
+    a.sim_warps = particle_blocks<k_batch_simulate<false, false, true>>(threads) * (unsigned)(threads / 32);
     k_batch_prepare<<<1, AWO_BATCH_MAX, 0, s>>>(a);
     if (total > 0) k_batch_starts<<<stream_blocks((int64_t)total, 256), 256, 0, s>>>(a);
     awo_status st = launch_status();
     bool after_particles = false;
-    for (int i = 0; i < n_req && st == AWO_OK; ++i) {
-        if (sim[i].N == 0u || sim[i].n_cells_max == 0u || sim[i].max_steps == 0u) continue;  // counted by the prologue
-        st = launch_particles(sim[i], threads, after_particles, s);
+    for (int r = 0; r < n_req && st == AWO_OK; ++r) {
+        SimArgs& c = own[r];
+        if (a.r[r].own_launch == OWN_NEVER || c.N == 0u || c.max_steps == 0u || a.r[r].n_cells_max == 0u) continue;
+        c.n_cells_dev = a.hdr->own_cells + r;
+        c.n_cells_max = a.r[r].n_cells_max;
+        c.next_item = &a.hdr->ws[r].next_item;
+        c.stats = a.stats + (size_t)a.r[r].id * a.stats_step;
+        c.starts = a.starts + a.r[r].starts_off;
+        c.group = b.group;
+        c.min_idle = b.min_idle;
+        c.check = &a.hdr->check;
+        st = launch_particles(c, threads, after_particles, s);
+        after_particles = true;
+    }
+    for (int kind = 0; kind < BATCH_KINDS && st == AWO_OK && total > 0; ++kind) {
+        b.first = kind_first[kind];
+        b.n = kind_first[kind + 1] - b.first;
+        b.kind = (uint32_t)kind;
+        if (b.n == 0u) continue;
+        if (b.n == 1u && a.r[b.first].own_launch == OWN_ALWAYS) continue;
+        auto launch = kind == 0 ? (plain ? launch_kind<false, true> : launch_kind<false, false>)
+                                : (plain ? launch_kind<true, true> : launch_kind<true, false>);
+        st = launch(b, threads, after_particles, s);
         after_particles = true;
     }
     if (st != AWO_OK) return st;

@@ -197,44 +197,11 @@ __global__ void __launch_bounds__(SIM_THREADS_MAX) k_simulate(const __grid_const
     }
 }
 
-// Shared memory asked for, in percent of an SM's 228 KB: the 64 KB split holds
-// the pools of all resident blocks, and the rest is L1.  Left to the driver,
-// instances got splits of 64 or 100 KB, and a launch with another split than
-// the one before it cannot start beside its last blocks (12 regions batched
-// 10.97 -> 9.92 ms, 2048^2 976 -> 968 us; asking for 100 KB 10.95 ms, for 32 KB,
-// 4 blocks an SM, 11.4 ms).
-constexpr int PARTICLE_CARVEOUT = 25;
-
-template <bool TEXELS, bool TEX, bool PLAIN, bool CHECK>
-static awo_status launch_instance(const SimArgs& a, int threads, bool early, cudaStream_t s)
-{
-    static int cached[64][3];  // resident blocks per SM, by device and block size (a race writes the same value)
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev < 0 || dev >= 64) dev = 0;
-    const size_t shared = (size_t)(threads / 32) * POOL_WORDS * sizeof(uint32_t);
-    int& per_sm = cached[dev][threads == 64 ? 0 : (threads == 128 ? 1 : 2)];
-    if (per_sm == 0) {
-        int b = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_simulate<TEXELS, TEX, PLAIN, CHECK>, threads, shared) !=
-                cudaSuccess ||
-            b < 1)
-            b = 1;
-        cudaFuncSetAttribute(k_simulate<TEXELS, TEX, PLAIN, CHECK>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             PARTICLE_CARVEOUT);
-        per_sm = b;
-    }
-    return launch_kernel(k_simulate<TEXELS, TEX, PLAIN, CHECK>, (unsigned)(sm_count() * per_sm + 1), (unsigned)threads, shared,
-                         early, s, a) == cudaSuccess
-               ? launch_status()
-               : AWO_ECUDA;
-}
-
 template <bool TEXELS, bool TEX, bool PLAIN>
 static awo_status launch_both(const SimArgs& a, int threads, bool after_particles, cudaStream_t s)
 {
-    const awo_status st = launch_instance<TEXELS, TEX, PLAIN, true>(a, threads, after_particles, s);
-    return st != AWO_OK ? st : launch_instance<TEXELS, TEX, PLAIN, false>(a, threads, true, s);
+    const awo_status st = launch_persistent<k_simulate<TEXELS, TEX, PLAIN, true>>(a, threads, after_particles, s);
+    return st != AWO_OK ? st : launch_persistent<k_simulate<TEXELS, TEX, PLAIN, false>>(a, threads, true, s);
 }
 
 awo_status launch_particles(const SimArgs& a, int threads, bool after_particles, cudaStream_t s)
