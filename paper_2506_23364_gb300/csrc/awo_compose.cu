@@ -59,11 +59,15 @@ __device__ __forceinline__ uint32_t compose_one(const RampSmem& r, const awo_col
 // the two blends.  `skip` (the colours of every value are finite): over a base, a
 // texel below count_min comes out as its base texel, 0 * colour + 1 * base, so
 // a group without a hit is copied.  Bound by issue where the map is hit (77%
-// of the slots) and by HBM elsewhere.  A thread's next group is loaded while it
-// works on this one: the branch alone left a fully hit raster 6% slower.  The
-// display pass of an 8192^2 map (velocity, mipmap, colours), a third of it hit:
-// 336.6 -> 319.1 us; all of it hit: 336.7 -> 337.3.
-template <int NS, bool HAS_BASE>
+// of the slots) and by HBM elsewhere.  AHEAD: a thread's next group is loaded
+// while it works on this one, which pays where the rasters come from HBM and
+// costs 6-16 registers (5 stops and a base 48 -> 54).  Times, us, over a base, a
+// third of the map hit / all of it (neither copies nor AHEAD; without AHEAD;
+// with it): 1024^2 4.8 / 4.9; 4.5 / 5.0; 4.9 / 5.4 -- 2496 x 1984 14.8 / 14.9; 10.6 /
+// 15.2; 11.7 / 16.2 -- 3001 x 2999 30.0 / 29.8; 25.4 / 30.5; 24.1 / 28.0 -- 8192^2 184 /
+// 184; 171 / 186; 159 / 177.  Without a base, without and with AHEAD: 2048^2 10.9;
+// 11.2 -- 3001 x 2999 24.4; 22.7 -- 8192^2 156; 143.
+template <int NS, bool HAS_BASE, bool AHEAD>
 __global__ void k_compose(const float* __restrict__ value, const uint32_t* __restrict__ count, int64_t n,
                           const __grid_constant__ awo_colormap cm, const uint8_t* __restrict__ base,
                           uint8_t* __restrict__ out, bool vec4, bool skip)
@@ -92,20 +96,19 @@ __global__ void k_compose(const float* __restrict__ value, const uint32_t* __res
             if (HAS_BASE) bn = __ldg(reinterpret_cast<const uint4*>(base32) + q);
         }
     };
-    fetch(tid);
+    if (AHEAD) fetch(tid);
     for (int64_t q = tid; q < n4; q += stride) {
+        if (!AHEAD) fetch(q);
         const float4 v = vn;
         const uint4 c = cn, b = bn;
-        fetch(q + stride);
-        if (HAS_BASE && skip && max(max(c.x, c.y), max(c.z, c.w)) < cm.count_min) {
-            reinterpret_cast<uint4*>(out32)[q] = b;
-            continue;
-        }
-        reinterpret_cast<uint4*>(out32)[q] =
-            make_uint4(compose_one<NS, HAS_BASE>(ramp, cm, v.x, c.x, b.x),
-                       compose_one<NS, HAS_BASE>(ramp, cm, v.y, c.y, b.y),
-                       compose_one<NS, HAS_BASE>(ramp, cm, v.z, c.z, b.z),
-                       compose_one<NS, HAS_BASE>(ramp, cm, v.w, c.w, b.w));
+        if (AHEAD) fetch(q + stride);
+        uint4 o = b;
+        if (!HAS_BASE || !skip || max(max(c.x, c.y), max(c.z, c.w)) >= cm.count_min)
+            o = make_uint4(compose_one<NS, HAS_BASE>(ramp, cm, v.x, c.x, b.x),
+                           compose_one<NS, HAS_BASE>(ramp, cm, v.y, c.y, b.y),
+                           compose_one<NS, HAS_BASE>(ramp, cm, v.z, c.z, b.z),
+                           compose_one<NS, HAS_BASE>(ramp, cm, v.w, c.w, b.w));
+        reinterpret_cast<uint4*>(out32)[q] = o;
     }
     for (int64_t i = 4 * n4 + tid; i < n; i += stride)
         out32[i] = compose_one<NS, HAS_BASE>(ramp, cm, value[i], count[i], HAS_BASE ? base32[i] : 0u);
@@ -115,21 +118,22 @@ template <int NS>
 static void launch_compose(const float* v, const uint32_t* c, int64_t n, const awo_colormap& cm, const uint8_t* b,
                            uint8_t* o, bool vec4, cudaStream_t s)
 {
-    // 42 registers: 5 blocks an SM are resident, so a grid of 8 per SM leaves a
-    // second, partial wave (8192^2 display pass: 8 -> 369 us, 32 -> 360, 128 ->
-    // 366); but each thread should have four groups or more (1984 x 2496: 34.8 us
-    // with four, 36.1 with one)
-    const int64_t groups = vec4 ? n / 4 + 1 : n;
-    const unsigned blocks = stream_blocks(groups, 256, groups >= (int64_t)sm_count() * 32 * 256 * 4
-                                                           ? 32
-                                                           : (groups >= (int64_t)sm_count() * 16 * 256 * 4 ? 16 : 8));
+    // Blocks an SM: few, so that a thread has several groups, but enough that the
+    // last, partial wave (4 or 5 blocks an SM are resident) is a small part.
+    // Without AHEAD, over a base, all hit, 8 / 16: 1400^2 7.3 / 7.6 us, 2048^2 13.6 /
+    // 13.2; with it 8 / 16 / 32: 3001 x 2999 28.0 / 28.5 / 31, 5003 x 4099 58.5 / 58.0 /
+    // 59.6, 8192^2 180 / 176 / 177 (a third hit, 16 stops, 189 / 171 / 164).
+    const int64_t groups = vec4 ? n / 4 + 1 : n, sm_threads = (int64_t)sm_count() * 256;
+    const bool ahead = groups >= sm_threads * 40;
+    const unsigned blocks =
+        ahead ? stream_blocks(groups, 256, groups >= sm_threads * 256 ? 32 : (groups >= sm_threads * 64 ? 16 : 8))
+              : stream_blocks(groups, 256, groups >= sm_threads * 24 ? 16 : 8);
     bool skip = true;
     for (int k = 0; k + 1 < NS; ++k)
         skip = skip && isfinite(cm.value[k]) && isfinite(cm.value[k + 1]) && isfinite(cm.value[k + 1] - cm.value[k]);
-    if (b)
-        k_compose<NS, true><<<blocks, 256, 0, s>>>(v, c, n, cm, b, o, vec4, skip);
-    else
-        k_compose<NS, false><<<blocks, 256, 0, s>>>(v, c, n, cm, b, o, vec4, skip);
+    auto kern = b ? (ahead ? k_compose<NS, true, true> : k_compose<NS, true, false>)
+                  : (ahead ? k_compose<NS, false, true> : k_compose<NS, false, false>);
+    kern<<<blocks, 256, 0, s>>>(v, c, n, cm, b, o, vec4, skip);
 }
 
 __device__ __forceinline__ float smooth_step(float e0, float e1, float x)
