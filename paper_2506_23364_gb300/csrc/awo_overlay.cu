@@ -57,7 +57,10 @@ __global__ void k_finalize(const float* __restrict__ maxe, int64_t n, float g2, 
 // one level-1 texel, so each is computed and written once.
 // Bound by HBM: 8192^2, velocity and a full chain 187 -> 166 us (984 MB, 88% of
 // the copy rate) with 16-byte loads, two level-1 texels a thread and row, where
-// rows are whole groups of four; 8-byte ones for other even rows.
+// rows are whole groups of four; 8-byte ones for other even rows.  Odd rows take
+// single cells, whose loads do not wait for one another: 5003 x 4099, 8 levels,
+// 68.4 -> 55.3 us (with a branch before each load the one texel a thread of the
+// second launch took 4.8 us; a kernel of its own, one texel a thread, 2.3).
 constexpr int LOD_TILE = 32;   // level-1 tile side
 constexpr int LOD_FUSED = 6;   // levels a block can finish: 32, 16, 8, 4, 2, 1
 
@@ -73,16 +76,6 @@ struct LodArgs {
     bool vec2;                               // level-0 child pairs as uint2 / float2
     bool vec4;                               // two of them as uint4 / float4, their results as uint2 / float2
 };
-
-template <bool FROM_MAXE>
-__device__ __forceinline__ float lod_vel0(const LodArgs& a, uint32_t i)
-{
-    const float x = __ldg(a.v0 + i);
-    if (!FROM_MAXE) return x;
-    const float v = __fsqrt_rn(__fmul_rn(a.g2, x));
-    a.vel0[i] = v;
-    return v;
-}
 
 template <bool FROM_MAXE>
 __device__ __forceinline__ float2 lod_vel0_pair(const LodArgs& a, uint32_t i)
@@ -173,20 +166,26 @@ __global__ void __launch_bounds__(256) k_lod_fused(const __grid_constant__ LodAr
                         m = fmaxf(m, fmaxf(v_1.x, v_1.y));
                     }
                 } else {
-                    sum = __ldg(a.c0 + r0);
-                    m = lod_vel0<FROM_MAXE>(a, r0);
-                    if (hx) {
-                        sum += __ldg(a.c0 + r0 + 1);
-                        m = fmaxf(m, lod_vel0<FROM_MAXE>(a, r0 + 1));
+                    // a child past the edge is the one before it again (the same maximum, not added), so that
+                    // no load waits for a branch
+                    const uint32_t i01 = r0 + (hx ? 1u : 0u), i10 = hy ? r1 : r0, i11 = i10 + (hx ? 1u : 0u);
+                    const uint32_t c00 = __ldg(a.c0 + r0), c01 = __ldg(a.c0 + i01), c10 = __ldg(a.c0 + i10),
+                                   c11 = __ldg(a.c0 + i11);
+                    float v00 = __ldg(a.v0 + r0), v01 = __ldg(a.v0 + i01), v10 = __ldg(a.v0 + i10),
+                          v11 = __ldg(a.v0 + i11);
+                    if (FROM_MAXE) {
+                        v00 = __fsqrt_rn(__fmul_rn(a.g2, v00));
+                        v01 = __fsqrt_rn(__fmul_rn(a.g2, v01));
+                        v10 = __fsqrt_rn(__fmul_rn(a.g2, v10));
+                        v11 = __fsqrt_rn(__fmul_rn(a.g2, v11));
+                        a.vel0[r0] = v00;
+                        if (hx) a.vel0[i01] = v01;
+                        if (hy) a.vel0[i10] = v10;
+                        if (hx && hy) a.vel0[i11] = v11;
                     }
-                    if (hy) {
-                        sum += __ldg(a.c0 + r1);
-                        m = fmaxf(m, lod_vel0<FROM_MAXE>(a, r1));
-                        if (hx) {
-                            sum += __ldg(a.c0 + r1 + 1);
-                            m = fmaxf(m, lod_vel0<FROM_MAXE>(a, r1 + 1));
-                        }
-                    }
+                    sum = (unsigned long long)c00 + (hx ? c01 : 0u) + (hy ? c10 : 0u);
+                    sum += hx && hy ? c11 : 0u;
+                    m = fmaxf(fmaxf(v00, v01), fmaxf(v10, v11));
                 }
                 const uint32_t c = saturated(sum);
                 const uint32_t o = (uint32_t)Y * (uint32_t)w1 + (uint32_t)X;
