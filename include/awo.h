@@ -261,15 +261,16 @@ awo_status awo_release_noalloc(const float* d_tan2, awo_grid g, double slope_lo_
  * 16-byte aligned (a work counter, the statistics, and a start record of up
  * to 32 bytes per release-list entry); contents undefined on entry and exit.
  * Gathers: on grids of at least 2^19 cells whose row pitch (4 * width bytes)
- * and d_h are aligned to the device's texture pitch alignment (32 bytes on
- * GB300), the particle kernel fetches each 2x2 footprint with one texture
+ * is aligned to the device's texture pitch alignment (32 bytes on GB300) and
+ * d_h to its texture alignment (512 bytes), the particle kernel fetches each
+ * 2x2 footprint with one texture
  * gather through a texture object that views d_h's 32-bit words (returned
  * bit for bit, subnormal heights included; clamp addressing, which is the
  * i1, j1 clamp above; indices and weights computed as stated).  The
  * object is created at the first call with that (d_h, width, height, device)
  * and kept for the life of the process, so that a captured CUDA graph keeps
- * a valid one; after 256 such buffers, further ones use plain loads, and a
- * call made while `stream` is being captured creates none (it uses an
+ * a valid one; after 256 such buffers of 2^20 cells or more, or 256 of fewer,
+ * further ones use plain loads, and a call made while `stream` is being captured creates none (it uses an
  * existing view, else the loads).  Both fetch the same heights: results do
  * not depend on the path.  The same holds for awo_simulate_batched (per
  * request) and the soft-deposit calls.
@@ -287,7 +288,8 @@ awo_status awo_simulate(const float* d_h, awo_grid g, const uint32_t* d_cells,
  * footprints of the W x H DEM at d_h by one texture gather through a texture
  * view of the buffer, 0 when they fetch them with four loads (grids under
  * 2^19 cells, a base address or row pitch off the texture alignment, 256
- * views already made, or `stream` being captured).  Like the first launch
+ * views already made of grids of its class, from 2^20 cells or below, or
+ * `stream` being captured).  Like the first launch
  * with that buffer, the call creates the view when one can be made.  Results
  * never depend on the path.  AWO_EINVAL: d_h or texture NULL, or a bad grid.
  */

@@ -253,10 +253,12 @@ void sim_constants(SimArgs& a, const float* d_h, awo_grid g, const awo_sim_param
 // object is a descriptor of (address, width, height, row pitch) -- no copy;
 // the words are viewed as 32-bit unsigned texels, returned bit for bit --
 // created on the first call with a buffer and kept for the life of the
-// process (at most DEM_VIEWS_MAX of them; further buffers take the load
-// path), so that a graph that captured a launch keeps a valid view.  A view
-// needs the row pitch and the base address aligned to the device's texture
-// pitch alignment and a grid within the 2D pitch-linear texture limits;
+// process (at most DEM_VIEWS_MAX of grids from DEM_VIEW_LARGE_CELLS and as
+// many of smaller ones, so that these, which gain less, never take a large
+// one's place; further buffers take the load path), so that a graph that
+// captured a launch keeps a valid view.  A view needs the row pitch and the base
+// address aligned to the device's texture pitch and texture alignments and a
+// grid within the 2D pitch-linear texture limits;
 // otherwise (or if creation fails) the kernel gathers with loads.  While the
 // launch stream is being captured into a graph no view is created (an
 // existing one is used, else the loads), so a capture never sees a call it
@@ -267,7 +269,7 @@ void sim_constants(SimArgs& a, const float* d_h, awo_grid g, const awo_sim_param
 // and 380 / 372, 81 / 77 (a DEM that small stays in L1, where the loads' latency
 // is shorter); 8192^2 5.5% less time.
 constexpr int DEM_VIEWS_MAX = 256;
-constexpr int64_t DEM_VIEW_MIN_CELLS = int64_t(1) << 19;
+constexpr int64_t DEM_VIEW_MIN_CELLS = int64_t(1) << 19, DEM_VIEW_LARGE_CELLS = int64_t(1) << 20;
 
 struct DemView {
     const float* h;
@@ -279,8 +281,11 @@ cudaTextureObject_t dem_texture(const float* d_h, awo_grid g, cudaStream_t s)
 {
     if (cells_of(g) < DEM_VIEW_MIN_CELLS) return 0;
     static std::mutex mu;
-    static DemView views[DEM_VIEWS_MAX];
-    static int n_views = 0;
+    static DemView tables[2][DEM_VIEWS_MAX];
+    static int used[2] = {0, 0};
+    const int large = cells_of(g) >= DEM_VIEW_LARGE_CELLS ? 1 : 0;
+    DemView* views = tables[large];
+    int& n_views = used[large];
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return 0;
     std::lock_guard<std::mutex> lock(mu);
@@ -293,13 +298,15 @@ cudaTextureObject_t dem_texture(const float* d_h, awo_grid g, cudaStream_t s)
         cudaGetLastError();
         return 0;
     }
-    int pitch_align = 0, max_w = 0, max_h = 0;
+    int pitch_align = 0, base_align = 0, max_w = 0, max_h = 0;
     if (cudaDeviceGetAttribute(&pitch_align, cudaDevAttrTexturePitchAlignment, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&base_align, cudaDevAttrTextureAlignment, dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&max_w, cudaDevAttrMaxTexture2DLinearWidth, dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&max_h, cudaDevAttrMaxTexture2DLinearHeight, dev) != cudaSuccess || pitch_align <= 0)
+        cudaDeviceGetAttribute(&max_h, cudaDevAttrMaxTexture2DLinearHeight, dev) != cudaSuccess || pitch_align <= 0 ||
+        base_align <= 0)
         return 0;
     const size_t pitch = (size_t)g.width * sizeof(float);
-    if ((pitch % (size_t)pitch_align) != 0 || ((uintptr_t)d_h % (uintptr_t)pitch_align) != 0 || g.width > max_w ||
+    if ((pitch % (size_t)pitch_align) != 0 || ((uintptr_t)d_h % (uintptr_t)base_align) != 0 || g.width > max_w ||
         g.height > max_h)
         return 0;
     cudaResourceDesc rd;
