@@ -398,7 +398,7 @@ extern "C" awo_status awo_simulate(const float* d_h, awo_grid g, const uint32_t*
     const bool work = a.N > 0 && n_cells_max > 0;
     if (work) {
         const unsigned pro_blocks = stream_blocks((int64_t)n_cells_max, 256);
-        if (launch_kernel(a.tg.texels ? k_sim_starts<true> : k_sim_starts<false>, pro_blocks, 256, 0, true, s, a) !=
+        if (launch_kernel(a.tg.texels ? k_sim_starts<true> : k_sim_starts<false>, pro_blocks, 256, 0, -1, true, s, a) !=
             cudaSuccess)
             return AWO_ECUDA;
     }
