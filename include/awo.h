@@ -256,7 +256,8 @@ awo_status awo_release_noalloc(const float* d_tan2, awo_grid g, double slope_lo_
  * n_cells_max.  d_count: uint32 [H*W], wraps modulo 2^32 (the call is
  * overflow-free whenever existing counts + n_traj + total_steps < 2^32).
  * d_maxe: float [H*W], non-negative (metres of energy-line height).
- * d_stats: awo_sim_stats on the device, overwritten (nullable).
+ * d_stats: awo_sim_stats on the device, overwritten at the end of the call's
+ * work (nullable).
  * Workspace: at least awo_simulate_workspace_bytes(n_cells_max) bytes,
  * 16-byte aligned (a work counter, the statistics, and a start record of up
  * to 32 bytes per release-list entry); contents undefined on entry and exit.
@@ -321,7 +322,8 @@ awo_status awo_simulate_time_kernel(void* ev_start, void* ev_stop);
  *    Rasters of different requests must not overlap.  The sum of n_cells_max
  *    over the requests must be < 2^31.
  *  - tuning: NULL for the default, or a configuration from awo_tune_batched.
- *  - d_stats: device array of n_req awo_sim_stats, overwritten (nullable).
+ *  - d_stats: device array of n_req awo_sim_stats, overwritten at the end of
+ *    the call's work (nullable).
  *  - Workspace: awo_simulate_batched_workspace_bytes(reqs, n_req) bytes,
  *    16-byte aligned, contents undefined on entry and exit.
  * The request table travels in the kernels' parameter blocks: the call makes

@@ -49,10 +49,11 @@ struct BatchReq {
 // or cells, footprints by texture or by loads.
 constexpr int BATCH_KINDS = 2;
 
-// Requests are in launch order (BatchArgs.r) but for the statistics of ws,
-// which are in the caller's.
+// Requests are in launch order (BatchArgs.r) but for the statistics, which are
+// in the caller's.
 struct BatchHeader {
-    SimWorkspace ws[AWO_BATCH_MAX];            // work counters (and statistics)
+    WorkCounter work[AWO_BATCH_MAX];
+    StatsCounters stats[AWO_BATCH_MAX];
     unsigned long long n_part[AWO_BATCH_MAX];  // particles of each request for k_batch_simulate
     uint32_t cell_prefix[AWO_BATCH_MAX + 1];   // start records before each request
     uint32_t unit_prefix[AWO_BATCH_MAX + 1];   // units of work before each request
@@ -75,8 +76,6 @@ struct BatchArgs {
     uint32_t sim_warps;           // warps of k_batch_simulate's launch
     unsigned long long look_min;  // look_paths of whole-cell steps
     BatchHeader* hdr;
-    unsigned long long* stats;  // 6 per request, stats_step words apart
-    uint32_t stats_step;
     TexelStart* starts;  // one 32-byte slot per release-list entry (CellStarts fill the first half of a request's)
 };
 static_assert(sizeof(BatchArgs) <= 32764, "the request table must fit the kernel parameter block");
@@ -102,8 +101,6 @@ struct BatchSimArgs {
     uint32_t group;      // particles a warp takes per fetch, 0: chosen by the kernel
     uint32_t min_idle;   // idle lanes a refill needs: 1, or 32 (lock-step batches)
     BatchHeader* hdr;
-    unsigned long long* stats;
-    uint32_t stats_step;
 };
 static_assert(sizeof(BatchSimArgs) <= 32764, "the request table must fit the kernel parameter block");
 
@@ -190,8 +187,8 @@ __global__ void __launch_bounds__(AWO_BATCH_MAX) k_batch_prepare(const __grid_co
         np = q.max_steps != 0u ? (unsigned long long)nc * q.N : 0ull;
         grid = q.n_grid;
         paths = (double)np / q.s;
-        a.hdr->ws[t] = SimWorkspace{};
-        for (int i = 0; i < 6; ++i) a.stats[(size_t)t * a.stats_step + i] = 0ull;
+        a.hdr->work[t] = WorkCounter{};
+        a.hdr->stats[t] = StatsCounters{};
     }
     const unsigned long long np_up = warp_inclusive(np), grid_up = warp_inclusive(grid);
     const double paths_up = warp_inclusive(paths);
@@ -258,7 +255,7 @@ __global__ void __launch_bounds__(256) k_batch_starts(const __grid_constant__ Ba
         }
         // particles of entries outside the grid are rejected; with max_steps = 0
         // every particle is capped at its release visit (no particle kernel work)
-        unsigned long long* st6 = a.stats + (size_t)q.id * a.stats_step;
+        unsigned long long* st6 = a.hdr->stats[q.id].n;
         if (!ok) atomicAdd(st6 + 5, (unsigned long long)q.N);
         if (ok && q.max_steps == 0u) {
             atomicAdd(st6 + 1, (unsigned long long)q.N);
@@ -310,7 +307,7 @@ __global__ void __launch_bounds__(256, 4) k_batch_simulate(const __grid_constant
             for (uint32_t k = 0u; k < a.n && i == a.n; k += 32u) {
                 const uint32_t j = min(k + lane, a.n - 1u), c = a.first + j;
                 const unsigned which =
-                    __ballot_sync(0xffffffffu, __ldcg(&a.hdr->ws[c].next_item) + 32ull * (prefix[j + 1u] - prefix[j]) <
+                    __ballot_sync(0xffffffffu, __ldcg(&a.hdr->work[c].next_item) + 32ull * (prefix[j + 1u] - prefix[j]) <
                                                    a.hdr->n_part[c]);
                 if (which) i = min(k + (uint32_t)__ffs(which) - 1u, a.n - 1u);
             }
@@ -319,7 +316,7 @@ __global__ void __launch_bounds__(256, 4) k_batch_simulate(const __grid_constant
         const uint32_t r = a.first + i;
         const BatchSimReq& q = a.r[r];
         const unsigned long long total = a.hdr->n_part[r];
-        unsigned long long* stats = a.stats + (size_t)q.id * a.stats_step;
+        unsigned long long* stats = a.hdr->stats[q.id].n;
         const uint32_t unit0 = prefix[i], units = prefix[i + 1] - unit0;
         if (units_left && g == unit0 && lane == 0u) {
             // particles of entries inside the grid (the prologue has counted the others)
@@ -332,9 +329,9 @@ __global__ void __launch_bounds__(256, 4) k_batch_simulate(const __grid_constant
         uint32_t chunk = share < a.hdr->chunk ? max((uint32_t)share & ~31u, 32u) : a.hdr->chunk;
         if (a.group) chunk = a.group;
         if (q.tex)
-            run_particles<TEXELS, 1, CHECK, PLAIN>(q, total, chunk, a.min_idle, &a.hdr->ws[r].next_item, stats, pool);
+            run_particles<TEXELS, 1, CHECK, PLAIN>(q, total, chunk, a.min_idle, &a.hdr->work[r].next_item, stats, pool);
         else
-            run_particles<TEXELS, 0, CHECK, PLAIN>(q, total, chunk, a.min_idle, &a.hdr->ws[r].next_item, stats, pool);
+            run_particles<TEXELS, 0, CHECK, PLAIN>(q, total, chunk, a.min_idle, &a.hdr->work[r].next_item, stats, pool);
         __syncwarp();  // the pool is empty; its words before the next request's
     }
 }
@@ -401,16 +398,10 @@ extern "C" awo_status awo_simulate_batched(const awo_sim_request* reqs, int32_t 
     a.look_min = look_paths(1.0f);
     a.hdr = static_cast<BatchHeader*>(d_ws);
     a.starts = reinterpret_cast<TexelStart*>(static_cast<char*>(d_ws) + BATCH_HEADER_BYTES);
-    // the kernels count into the caller's statistics where they can
-    const bool direct = d_stats && (((uintptr_t)d_stats) & 7u) == 0;
-    a.stats = direct ? reinterpret_cast<unsigned long long*>(d_stats) : a.hdr->ws[0].stats;
-    a.stats_step = (uint32_t)((direct ? sizeof(awo_sim_stats) : sizeof(SimWorkspace)) / sizeof(unsigned long long));
     // the requests by kind, each kind's in the caller's order
     BatchSimArgs b;
     memset(&b, 0, sizeof(b));
     b.hdr = a.hdr;
-    b.stats = a.stats;
-    b.stats_step = a.stats_step;
     b.group = tuning ? (uint32_t)tuning->group_particles : 0u;
     b.min_idle = tuning && tuning->refill == AWO_REFILL_WARP ? 32u : 1u;
     bool plain = true;
@@ -485,8 +476,8 @@ extern "C" awo_status awo_simulate_batched(const awo_sim_request* reqs, int32_t 
         if (a.r[r].own_launch == OWN_NEVER || c.N == 0u || c.max_steps == 0u || a.r[r].n_cells_max == 0u) continue;
         c.n_cells_dev = a.hdr->own_cells + r;
         c.n_cells_max = a.r[r].n_cells_max;
-        c.next_item = &a.hdr->ws[r].next_item;
-        c.stats = a.stats + (size_t)a.r[r].id * a.stats_step;
+        c.next_item = &a.hdr->work[r].next_item;
+        c.stats = a.hdr->stats[a.r[r].id].n;
         c.starts = a.starts + a.r[r].starts_off;
         c.group = b.group;
         c.min_idle = b.min_idle;
@@ -506,10 +497,7 @@ extern "C" awo_status awo_simulate_batched(const awo_sim_request* reqs, int32_t 
         after_particles = true;
     }
     if (st != AWO_OK) return st;
-    if (d_stats && !direct &&
-        cudaMemcpy2DAsync(d_stats, sizeof(awo_sim_stats), a.hdr->ws[0].stats, sizeof(SimWorkspace), sizeof(awo_sim_stats),
-                          (size_t)n_req, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
-        return AWO_ECUDA;
+    if (d_stats) return publish_stats(a.hdr->stats, d_stats, n_req, after_particles, s);
     return AWO_OK;
 }
 

@@ -70,10 +70,10 @@ __device__ __forceinline__ uint32_t release_count(const SimArgs& a)
 
 // Start of a call: the work counter and the statistics zeroed, and n words of
 // both rasters (CLEAR_OUTPUTS; 0 otherwise) -- one launch where three memsets
-// and, for the statistics, a copy at the end of the call took four (2 us each
-// between the kernels of a small call; at 8192^2 as fast as the memsets).
+// took three (2 us each between the kernels of a small call; at 8192^2 as fast
+// as the memsets).
 __global__ void __launch_bounds__(256) k_sim_clear(uint32_t* __restrict__ count, uint32_t* __restrict__ maxe, int64_t n,
-                                                   SimWorkspace* ws, unsigned long long* stats, bool vec4)
+                                                   SimWorkspace* ws, bool vec4)
 {
     asm volatile("griddepcontrol.launch_dependents;");
     const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
@@ -84,8 +84,28 @@ __global__ void __launch_bounds__(256) k_sim_clear(uint32_t* __restrict__ count,
         reinterpret_cast<uint4*>(maxe)[q] = zero;
     }
     for (int64_t i = 4 * n4 + tid; i < n; i += stride) count[i] = maxe[i] = 0u;
-    if (tid < 6) ws->stats[tid] = stats[tid] = 0ull;
-    if (tid == 6) ws->next_item = 0ull;
+    if (tid < 6) ws->stats.n[tid] = 0ull;
+    if (tid == 6) ws->work.next_item = 0ull;
+}
+
+// End of a call: request blockIdx.x's statistics to the caller's array, byte
+// by byte (of any alignment).  The kernels count in the workspace, so that the
+// array holds the last call's statistics until this one's are complete.
+__global__ void __launch_bounds__(64) k_sim_publish(const StatsCounters* from, unsigned char* stats)
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // the particle kernel
+    const unsigned i = threadIdx.x;
+    if (i < sizeof(awo_sim_stats))
+        stats[(size_t)blockIdx.x * sizeof(awo_sim_stats) + i] =
+            reinterpret_cast<const unsigned char*>(from[blockIdx.x].n)[i];
+}
+
+awo_status publish_stats(const StatsCounters* from, awo_sim_stats* d_stats, int n, bool early, cudaStream_t s)
+{
+    return launch_kernel(k_sim_publish, (unsigned)n, 64u, 0, -1, early, s, from,
+                         reinterpret_cast<unsigned char*>(d_stats)) == cudaSuccess
+               ? launch_status()
+               : AWO_ECUDA;
 }
 
 // Prologue: per release-list entry, the start record (at its slot in the
@@ -337,7 +357,7 @@ cudaTextureObject_t dem_texture(const float* d_h, awo_grid g, cudaStream_t s)
 
 using namespace awo;
 
-static size_t starts_offset() { return 256; }
+static size_t starts_offset() { return (sizeof(SimWorkspace) + 255) / 256 * 256; }
 
 // Events of awo_simulate_time_kernel for the next awo_simulate of this thread.
 static thread_local cudaEvent_t t_kernel_events[2] = {nullptr, nullptr};
@@ -376,22 +396,20 @@ extern "C" awo_status awo_simulate(const float* d_h, awo_grid g, const uint32_t*
     if (ws_bytes < awo_simulate_workspace_bytes(n_cells_max)) return AWO_ENOMEM;
     cudaStream_t s = as_stream(stream);
     SimWorkspace* ws = static_cast<SimWorkspace*>(d_ws);
-    // the kernels count into the caller's statistics where they can
-    const bool direct = d_stats && (((uintptr_t)d_stats) & 7u) == 0;
 
     SimArgs a;
     sim_constants(a, d_h, g, p, d_count, d_maxe, s);
     a.cells = d_cells;
     a.n_cells_dev = d_n_cells;
     a.n_cells_max = n_cells_max;
-    a.next_item = &ws->next_item;
-    a.stats = direct ? reinterpret_cast<unsigned long long*>(d_stats) : ws->stats;
+    a.next_item = &ws->work.next_item;
+    a.stats = ws->stats.n;
     a.starts = static_cast<char*>(d_ws) + starts_offset();
 
     const int64_t n_clear = (p->flags & AWO_SIM_CLEAR_OUTPUTS) ? cells_of(g) : 0;
     const bool vec4 = ((((uintptr_t)d_count) | ((uintptr_t)d_maxe)) & 15u) == 0;
     k_sim_clear<<<stream_blocks(vec4 ? n_clear / 4 : n_clear, 256), 256, 0, s>>>(
-        d_count, reinterpret_cast<uint32_t*>(d_maxe), n_clear, ws, a.stats, vec4);
+        d_count, reinterpret_cast<uint32_t*>(d_maxe), n_clear, ws, vec4);
     awo_status st = launch_status();
     if (st != AWO_OK) return st;
 
@@ -408,8 +426,6 @@ extern "C" awo_status awo_simulate(const float* d_h, awo_grid g, const uint32_t*
         if (st != AWO_OK) return st;
     }
     if (ev_stop && cudaEventRecord(ev_stop, s) != cudaSuccess) return AWO_ECUDA;
-    if (d_stats && !direct && cudaMemcpyAsync(d_stats, ws->stats, sizeof(awo_sim_stats), cudaMemcpyDeviceToDevice, s) !=
-                                  cudaSuccess)
-        return AWO_ECUDA;
+    if (d_stats) return publish_stats(&ws->stats, d_stats, 1, ev_stop == nullptr, s);
     return AWO_OK;
 }
