@@ -306,6 +306,20 @@ def _cpu_baseline(w, seconds: float, threads: int | None = None) -> dict:
 # ----------------------------------------------------------------------------
 # arms
 # ----------------------------------------------------------------------------
+def launches_per_step(awo, width: int, height: int, release_log2: int, levels: int) -> int:
+    """Kernels that one Overlay.run launches."""
+    texels = width * height
+    if release_log2:
+        wr, hr = awo.awo_release_texture_dims(awo.grid(width, height, 1.0), release_log2)
+        texels = wr * hr
+    # decode, normals and release mask (one launch; two with a release texture), scan above 4096 tiles of 4096
+    # texels, scatter
+    terrain = 1 + (release_log2 != 0) + (-(-texels // 4096) > 4096) + 1
+    simulate = 5  # clear, prologue, the particle kernel's two instances (one of them ends at once), statistics
+    overlay = max(1, -(-(levels - 1) // 6))  # velocity and six levels, then six further levels a launch
+    return terrain + simulate + overlay
+
+
 def run_awo(args, R: Ranks):
     import numpy as np
     import torch
@@ -339,12 +353,7 @@ def run_awo(args, R: Ranks):
     torch.cuda.synchronize()
     st = ov.stats_dict()
     visits = st["total_steps"] + st["n_traj"]
-    # decode, normals and release mask (one launch), scatter (and a scan of its own above 4096 tiles of 4096
-    # cells), clear, particle prologue and the particle kernel's two instances (one of them ends at once), then
-    # velocity and mipmap: one launch for both and six levels, one per six further levels (velocity alone
-    # without a mipmap)
-    lod_launches = max(1, -(-(w.lod_levels - 1) // 6))
-    launches_per_step = 1 + 1 + (w.width * w.height > 4096 * 4096) + 4 + lod_launches
+    per_step = launches_per_step(awo, w.width, w.height, args.release_log2, w.lod_levels)
 
     peaks_probe = _probe_peaks(torch, awo)
     clocks = ClockSampler(R.local)
@@ -428,7 +437,7 @@ def run_awo(args, R: Ranks):
             "simulate_steps_per_s": st["total_steps"] / (sim_ms / 1e3),
             "particles_per_s": st["n_traj"] / (sim_ms / 1e3), "stats": st,
             "e2e": e2e,
-            "gpu_launches": launches_per_step * args.steps, "roofline": roofline, "roofline_l2": l2,
+            "gpu_launches": per_step * args.steps, "roofline": roofline, "roofline_l2": l2,
             "roofline_hbm": roofline_hbm,
             "clocks": clk, "kernel_sha": sha}
     if R.rank == 0 and R.world == 1 and not args.no_cpu_baseline and not args.release_log2:
