@@ -123,15 +123,23 @@ constexpr uint32_t CHUNKS_PER_WARP = 32;  // fetches a warp makes on an even spl
 // Requests with a launch of k_simulate each: their constants are then at
 // fixed places of the parameter block, which runs up to 167 G moves/s where
 // k_batch_simulate, issue-bound, ends at 140; but a launch leaves the GPU
-// partly idle at its end, and costs the host 7 us.  4 regions of 2048^2: 24 M
-// particles each 6.02 against 7.36 ms, 6 M each 2.80 against 2.10; 12 of 1280^2,
-// 5.9 M each, 7.7 against 5.8; 12 of 512^2..2048^2 7.97 with the line at 6 M, 8.14
-// at 10 M, 8.47 without launches of their own (7.75 with one for each).  The
-// number of particles is known on the device alone, so the host launches for
-// every request that can have LARGE_PARTICLES at the share of release cells
-// that steep terrain has (1 in 22), and the launch ends at once when there are
-// fewer.  A request that is alone of its kind has its own launch, too.
-constexpr unsigned long long LARGE_PARTICLES = 6000000ull, LARGE_MOST = 22ull * LARGE_PARTICLES;
+// partly idle at its end, and costs the host 4 us.  Only the instance with the
+// look is launched, so they need a batch for which looking pays: a second
+// launch's 1500 blocks, which end at once, had to trickle through the few
+// slots that the first one's last particles left free.  Their warps take
+// OWN_CHUNK particles a fetch or more: with 32, fetches at the one counter
+// held them back.  12 of 1280^2, 5.7 M particles each: 5.74 ms together, 7.66
+// with two launches each, 5.67 with one, 5.27 with one and 128 a fetch (96 5.29,
+// 256 5.38); 4 of 2048^2, 23 M each, 7.4 together, 6.03 so; 16 of 1024^2, 2.9 M
+// each, 3.52 together, 3.33 with launches of their own, 4.4 M each 5.27 and 4.59;
+// 12 of 512^2..2048^2 7.35 (8.47 all together, 7.75 with two launches each).
+// The number of particles is known on the device alone, so the host launches
+// for every request that can have LARGE_PARTICLES at the share of release
+// cells that steep terrain has (1 in 22), and the launch ends at once when
+// there are fewer (32 of 2048^2 with few release cells: 2.38 -> 2.47 ms).  A
+// request that is alone of its kind has its own launch, too.
+constexpr unsigned long long LARGE_PARTICLES = 3000000ull, LARGE_MOST = 22ull * LARGE_PARTICLES;
+constexpr uint32_t OWN_CHUNK = 128;
 enum OwnLaunch : uint32_t { OWN_NEVER, OWN_IF_LARGE, OWN_ALWAYS };
 
 // Index r with prefix[r] <= g < prefix[r+1] (prefix has n + 1 entries).
@@ -197,8 +205,13 @@ __global__ void __launch_bounds__(AWO_BATCH_MAX) k_batch_prepare(const __grid_co
     unsigned long long total = 0ull;
 #pragma unroll
     for (int w = 0; w < WARPS; ++w) total += s_total[w];
+    unsigned long long grids = 0ull;
+    double sum_paths = 0.0;
+#pragma unroll
+    for (int w = 0; w < WARPS; ++w) grids += s_grid[w], sum_paths += s_paths[w];
+    const bool check = sum_paths >= (double)a.look_min || total >= 7ull * grids;  // as check_pays
     const bool own = mine && (a.r[t].own_launch == OWN_ALWAYS ||
-                              (a.r[t].own_launch == OWN_IF_LARGE && np >= LARGE_PARTICLES));
+                              (a.r[t].own_launch == OWN_IF_LARGE && check && np >= LARGE_PARTICLES));
     // FP32 is enough to share out the work (a 64-bit division costs more than the rest of this kernel)
     const float warps = (float)a.sim_warps, unit = fmaxf((float)total / (warps * UNITS_PER_WARP), 32.0f);
     const float least = fminf((float)np / 32.0f, warps / REQUESTS_IN_FLIGHT);
@@ -216,12 +229,8 @@ __global__ void __launch_bounds__(AWO_BATCH_MAX) k_batch_prepare(const __grid_co
     a.hdr->unit_prefix[t + 1] = units1;
     if (t == 0) {
         a.hdr->cell_prefix[0] = a.hdr->unit_prefix[0] = 0u;
-        unsigned long long grids = 0ull;
-        double sum_paths = 0.0;
-#pragma unroll
-        for (int w = 0; w < WARPS; ++w) grids += s_grid[w], sum_paths += s_paths[w];
         a.hdr->chunk = max((uint32_t)fminf((float)total / (warps * CHUNKS_PER_WARP), 1024.0f) & ~31u, 32u);
-        a.hdr->check = sum_paths >= (double)a.look_min || total >= 7ull * grids ? 1u : 0u;  // as check_pays
+        a.hdr->check = check ? 1u : 0u;
     }
 }
 
@@ -482,7 +491,8 @@ extern "C" awo_status awo_simulate_batched(const awo_sim_request* reqs, int32_t 
         c.group = b.group;
         c.min_idle = b.min_idle;
         c.check = &a.hdr->check;
-        st = launch_particles(c, threads, after_particles, s);
+        c.least_chunk = a.r[r].own_launch == OWN_IF_LARGE ? OWN_CHUNK : 32u;
+        st = launch_particles(c, threads, after_particles, a.r[r].own_launch == OWN_IF_LARGE, s);
         after_particles = true;
     }
     for (int kind = 0; kind < BATCH_KINDS && st == AWO_OK && total > 0; ++kind) {

@@ -210,7 +210,7 @@ __global__ void __launch_bounds__(SIM_THREADS_MAX) k_simulate(const __grid_const
         // particles a warp takes per fetch: a multiple of 32 in [32,
         // SIM_CHUNK_MAX], about total / (warps * SIM_CHUNKS_PER_WARP)
         const unsigned long long even = total / ((unsigned long long)blocks * (blockDim.x >> 5) * SIM_CHUNKS_PER_WARP);
-        uint32_t chunk = even > SIM_CHUNK_MAX ? SIM_CHUNK_MAX : max((uint32_t)even & ~31u, 32u);
+        uint32_t chunk = even > SIM_CHUNK_MAX ? SIM_CHUNK_MAX : max((uint32_t)even & ~31u, a.least_chunk);
         if (a.group) chunk = a.group;
         run_particles<TEXELS, TEX ? 1 : 0, CHECK, PLAIN>(a, total, chunk, a.min_idle, a.next_item, a.stats,
                                                   s_pool + warp * POOL_WORDS);
@@ -218,20 +218,20 @@ __global__ void __launch_bounds__(SIM_THREADS_MAX) k_simulate(const __grid_const
 }
 
 template <bool TEXELS, bool TEX, bool PLAIN>
-static awo_status launch_both(const SimArgs& a, int threads, bool after_particles, cudaStream_t s)
+static awo_status launch_both(const SimArgs& a, int threads, bool after_particles, bool look, cudaStream_t s)
 {
     const awo_status st = launch_persistent<k_simulate<TEXELS, TEX, PLAIN, true>>(a, threads, after_particles, s);
-    return st != AWO_OK ? st : launch_persistent<k_simulate<TEXELS, TEX, PLAIN, false>>(a, threads, true, s);
+    return st != AWO_OK || look ? st : launch_persistent<k_simulate<TEXELS, TEX, PLAIN, false>>(a, threads, true, s);
 }
 
-awo_status launch_particles(const SimArgs& a, int threads, bool after_particles, cudaStream_t s)
+awo_status launch_particles(const SimArgs& a, int threads, bool after_particles, bool look, cudaStream_t s)
 {
     const bool plain = a.s == 1.0f && a.kD == 0.0f;
     auto launch = a.tg.texels ? (a.tex ? (plain ? launch_both<true, true, true> : launch_both<true, true, false>)
                                        : (plain ? launch_both<true, false, true> : launch_both<true, false, false>))
                               : (a.tex ? (plain ? launch_both<false, true, true> : launch_both<false, true, false>)
                                        : (plain ? launch_both<false, false, true> : launch_both<false, false, false>));
-    return launch(a, threads, after_particles, s);
+    return launch(a, threads, after_particles, look, s);
 }
 
 void sim_constants(SimArgs& a, const float* d_h, awo_grid g, const awo_sim_params* p, uint32_t* d_count, float* d_maxe,
@@ -266,6 +266,7 @@ void sim_constants(SimArgs& a, const float* d_h, awo_grid g, const awo_sim_param
     a.tg.texels = p->release_log2 != 0 ? 1u : 0u;
     a.tex = dem_texture(d_h, g, s);
     a.min_idle = 1u;
+    a.least_chunk = 32u;
     a.look_min = look_paths(p->step_scale);
 }
 
@@ -422,7 +423,7 @@ extern "C" awo_status awo_simulate(const float* d_h, awo_grid g, const uint32_t*
     }
     if (ev_start && cudaEventRecord(ev_start, s) != cudaSuccess) return AWO_ECUDA;
     if (work && a.max_steps != 0u) {  // else every particle is capped at its release visit
-        st = launch_particles(a, SIM_THREADS, false, s);
+        st = launch_particles(a, SIM_THREADS, false, false, s);
         if (st != AWO_OK) return st;
     }
     if (ev_stop && cudaEventRecord(ev_stop, s) != cudaSuccess) return AWO_ECUDA;

@@ -14,7 +14,7 @@ from paper_2506_23364_gb300 import inputs
 
 pytestmark = pytest.mark.gpu
 
-LARGE = 6_000_000  # particles from which a request has a launch of its own
+LARGE = 3_000_000  # particles from which a request has a launch of its own, in a batch that looks at the maxima
 
 
 class Region:
@@ -109,13 +109,17 @@ def test_numbers_of_requests(n):
     _run(regions)
 
 
+@pytest.mark.parametrize("look", [False, True])
 @pytest.mark.parametrize("n_cells", [LARGE // 256, LARGE // 256 + 1])
-def test_either_side_of_a_launch_of_its_own(n_cells):
+def test_either_side_of_a_launch_of_its_own(n_cells, look):
     dem = _slope(512, 1024, 2)
     kw = dict(traj_per_cell=256, max_steps=2)
-    big = [Region(dem, (np.arange(n_cells) * 22) % dem.size, dict(kw, seed=i), n_max=dem.size) for i in range(2)]
+    lanes = 1280 * torch.cuda.get_device_properties(0).multi_processor_count
+    n_big = 3 if look else 2
+    big = [Region(dem, (np.arange(n_cells) * 22) % dem.size, dict(kw, seed=i), n_max=dem.size) for i in range(n_big)]
     small = [Region(_slope(64, 64, i), np.arange(0, 4096, 9), dict(traj_per_cell=20, max_steps=90, seed=i)) for i in range(2)]
-    _run([big[0], small[0], big[1], small[1]])
+    assert (sum(q.n * q.kw["traj_per_cell"] for q in big + small) >= 32 * lanes) == look
+    _run([*big[:1], small[0], *big[1:], small[1]])
 
 
 def test_against_the_oracle():
