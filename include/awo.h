@@ -74,8 +74,8 @@ typedef struct {
                           /* 0: the list holds DEM cells                               */
 } awo_sim_params;
 
-/* awo_sim_params.flags: clear d_count and d_maxe (cudaMemsetAsync on the
- * stream) before the particles run, instead of accumulating into them. */
+/* awo_sim_params.flags: clear d_count and d_maxe on the
+ * stream before the particles run, instead of accumulating into them. */
 #define AWO_SIM_CLEAR_OUTPUTS 1u
 
 /* Statistics of one awo_simulate call (device layout, 6 x uint64). */

@@ -38,7 +38,7 @@
 //  * Arithmetic is FP32 with explicit round-to-nearest intrinsics: no fused
 //    multiply-add that changes a rounding, IEEE sqrt and reciprocal, so every
 //    particle follows the formulas of awo.h bit for bit.
-//  * What bounds it: issue on the 8192^2 workload (82% of issue slots; 151
+//  * What bounds it: issue on the 8192^2 workload (82% of issue slots; 145-150
 //    warp instructions per move of a warp, from 222), the visits' traffic to
 //    the L2 and the footprint gathers' latency on the long-trajectory ones
 //    (2048^2: 73% of issue slots, L2 62%, from 67% and 72%).  Measured and not
@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(256) k_sim_starts(const __grid_constant__ SimA
 // or with the choice as a predicate, the 8192^2 workload took 2% more).
 //
 // Every launch lets the next one start as soon as its blocks are resident
-// (programmatic dependent launch), so the blocks of a batch's next request
+// (programmatic dependent launch), so the blocks of a batch's next launch
 // fill the SMs as this one's warps run out of particles.  The last block of a
 // launch does nothing but wait for the launch before it, so that a launch is
 // complete only when all before it are, and what follows on the stream is

@@ -84,10 +84,10 @@ constexpr uint32_t SOFT_REFILL_IDLE = 4;
 
 // Soft particles, GRAD = false: deposits; GRAD = true: gradient sums.  TEX:
 // footprints by texture gather through a.tex (else by loads).  Persistent,
-// one lane per particle, with the lane refill of the particle kernels
-// (awo_simulate.cu): a warp takes chunks of consecutive particles (entry,
-// then particle j) and restarts a lane whose particle has ended, so a long
-// particle does not keep the other lanes of its warp idle.  Each loop
+// one lane per particle: a warp takes chunks of consecutive particles (entry,
+// then particle j) and restarts a lane whose particle has ended with the next
+// one, so a long particle does not keep the other lanes of its warp idle (no
+// fresh pairs and no pool, as run_particles has).  Each loop
 // iteration is two moves from one Philox block (moves n and n + 1 take words
 // 0-1 and 2-3 of block n >> 1; lanes start at n = 0 and move in pairs).  Per
 // particle the arithmetic is that of the hard mode's moves plus the
@@ -225,7 +225,7 @@ __global__ void __launch_bounds__(SOFT_THREADS, GRAD ? 8 : 9) k_soft(const __gri
     };
 
     while (true) {
-        // ---- refill idle lanes (as in k_simulate) ----
+        // ---- refill idle lanes ----
         const unsigned idle = __ballot_sync(0xffffffffu, !live);
         idle_acc += (uint32_t)__popc(idle);
         if (idle != 0u && idle_acc >= SOFT_REFILL_IDLE && !exhausted) {

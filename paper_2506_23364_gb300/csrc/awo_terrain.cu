@@ -1246,10 +1246,6 @@ extern "C" awo_status awo_release_texture(const float* d_tan2, awo_grid g, int32
     // float4 reads of tan2 rows: base 16-byte aligned and W a multiple of 4,
     // so that every row and every run start (a multiple of 16 / 2^r cells) is
     const bool vec = (((uintptr_t)d_tan2) & 15u) == 0 && (g.width & 3) == 0;
-    auto kern = release_log2 == 0   ? (vec ? k_release_texture_mask<0, true> : k_release_texture_mask<0, false>)
-                : release_log2 == 1 ? (vec ? k_release_texture_mask<1, true> : k_release_texture_mask<1, false>)
-                : release_log2 == 2 ? (vec ? k_release_texture_mask<2, true> : k_release_texture_mask<2, false>)
-                                    : k_release_texture_mask<3, false>;
     if ((release_log2 == 1 || release_log2 == 2) && g.height >= 2 && g.height < 65535 && wr % RT_TILE == 0) {
         // rows are whole tiles: one launch of row groups that share their tan^2 rows
         const dim3 grid((unsigned)(wr / RT_TILE), (unsigned)g.height + 1u);  // at most 65535 groups
@@ -1272,6 +1268,10 @@ extern "C" awo_status awo_release_texture(const float* d_tan2, awo_grid g, int32
         k_release_texture_texels<<<tiles, NC_THREADS, 0, s>>>(d_tan2, g.width, g.height, (uint32_t)wr, (uint32_t)n, scale,
                                                               t_lo, t_hi, d_mask, tile_count);
     } else {
+        auto kern = release_log2 == 0   ? (vec ? k_release_texture_mask<0, true> : k_release_texture_mask<0, false>)
+                    : release_log2 == 1 ? (vec ? k_release_texture_mask<1, true> : k_release_texture_mask<1, false>)
+                    : release_log2 == 2 ? (vec ? k_release_texture_mask<2, true> : k_release_texture_mask<2, false>)
+                                        : k_release_texture_mask<3, false>;
         kern<<<tiles, RT_THREADS, 0, s>>>(d_tan2, g.width, g.height, (uint32_t)wr, n, scale, t_lo, t_hi, d_mask,
                                           tile_count);
     }
