@@ -67,9 +67,9 @@ ALG_OPS_PER_VISIT = 126
 #   atomic_busy: lts__d_atomic_input_cycles_active.avg.pct_of_peak_sustained_elapsed
 #     / 100, the share of cycles the L2's reduction units take input
 KERNEL_COUNTERS: dict[str, dict[str, float]] = {
-    "98baa25ce7c2d225": {"dram": (1138.118912e6 + 177.382144e6) / 1754008332, "lts_frac": 0.5105,
-                         "red_sectors": 1191971881 / 1754008332, "read_sectors": 38551609 / 1754008332,
-                         "atomic_busy": 0.3353},
+    "cd33adc2e6fd6334": {"dram": (1137.729792e6 + 177.523200e6) / 1754008332, "lts_frac": 0.5134,
+                         "red_sectors": 1191977153 / 1754008332, "read_sectors": 42019872 / 1754008332,
+                         "atomic_busy": 0.3367},
 }
 
 

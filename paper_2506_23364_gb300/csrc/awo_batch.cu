@@ -109,14 +109,16 @@ static_assert(sizeof(BatchSimArgs) <= 32764, "the request table must fit the ker
 // until none is left to take.  The batch has UNITS_PER_WARP units for each
 // warp of the launch, split over the requests by their particles, so that
 // some requests are always at work while another one's last particles run
-// out; but the warps of an SM that work on many requests keep pushing one
-// another's constants out of the constant cache, so a request gets at least
-// one in REQUESTS_IN_FLIGHT of the warps (or one for every 32 of its
-// particles).  A warp that finds no unit left joins a request that has more
-// particles waiting than its own warps take next.  Measured (ms; 128 regions
-// of 256^2 with 64 particles per release cell / 32 of 1024^2 with 32): 1 unit a
-// warp and no least share 7.0 / 8.6, 2 and the share of 1 in 8 2.77 / 3.84, all
-// warps on every request in turn 4.0 / 5.8.
+// out.  But warps wait for their requests' constants when an SM works on many
+// requests (the stall on indexed constant loads is 1.3 warps an issue with the
+// shares below, 20.8 without a least share), so a request gets at least one in
+// REQUESTS_IN_FLIGHT of the warps (or one for every 32 of its particles).  A
+// warp that finds no unit left joins a request that has more particles
+// waiting than its own warps take next.  Measured (ms; 128 regions of 256^2 with
+// 64 particles per release cell / 128 of 512^2 with 16 / 32 of 1024^2 with 32), 2
+// units a warp and a share of 1 in 8: 2.76 / 2.81 / 3.87; 1 in 32 3.45 / 3.29 / 4.19;
+// no least share 4.14 / 3.99 / 4.19, with 1 unit a warp 4.95 / 4.77 / 6.45; all warps
+// on each request in turn 3.89 / 4.57 / 4.12.
 constexpr uint32_t UNITS_PER_WARP = 2, REQUESTS_IN_FLIGHT = 8;
 constexpr uint32_t CHUNKS_PER_WARP = 32;  // fetches a warp makes on an even split (16: 12 of 1280^2 5.80 -> 5.95 ms)
 
@@ -277,13 +279,13 @@ __global__ void __launch_bounds__(256) k_batch_starts(const __grid_constant__ Ba
 // of the two ends at once, as in k_simulate).  Persistent; the last block
 // orders the launch after the one before it (see k_simulate).
 //
-// A request's constants are read from the parameter block through an index
-// that the compiler knows to be the same for the whole warp (it comes from
-// ballots): held in a lane's registers they took 62-92 of them.  64 registers,
-// 8 blocks an SM: 48 (and 16 bytes spilled) gave 2% more on large requests and
-// took 5-8% longer on small ones, which are bound by latency.  128 regions of
-// 64^2 1.44 -> 0.85 ms against a launch for each, of 512^2 with 16 particles per
-// release cell 5.43 -> 2.85, 32 of 1024^2 with 32 6.05 -> 3.84.
+// A request's constants are read where they are used, by constant loads
+// indexed with the request (11% of the instructions): held in a lane's
+// registers they took 62-92 of them.  64 registers, 8 blocks an SM: 48 (and 16
+// bytes spilled) gave 2% more on large requests and took 5-8% longer on small
+// ones, which are bound by latency.  128 regions of 64^2 1.44 -> 0.85 ms against a
+// launch for each, of 512^2 with 16 particles per release cell 5.43 -> 2.85, 32 of
+// 1024^2 with 32 6.05 -> 3.84.
 template <bool TEXELS, bool PLAIN, bool CHECK>
 __global__ void __launch_bounds__(256, 4) k_batch_simulate(const __grid_constant__ BatchSimArgs a)
 {
